@@ -22,6 +22,7 @@
 #include "lgf_gstep.cuh"
 #include "lgf_kernels.cuh"
 #include "lgf_reduce.cuh"
+#include "lgf_stage.cuh"
 
 namespace lgf {
 
@@ -165,19 +166,10 @@ __global__ void __launch_bounds__(kStageMats) k_materialize(const cx<T>* __restr
     M3<T> w, r;
     mm<T, 3>(w, gx, u);
     mm_dag<T, 3>(r, w, gf);
-    double* d = sm + threadIdx.x * kStagePitch;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      d[2 * q] = (double)r.e[q / 3][q % 3].re;
-      d[2 * q + 1] = (double)r.e[q / 3][q % 3].im;
-    }
+    stage_matrix(sm, r);
   }
   __syncthreads();
-  double2* dst = reinterpret_cast<double2*>(aos + first * 18);
-  for (int j = threadIdx.x; j < n * 9; j += blockDim.x) {
-    const int m = (2 * j) / 18, k = (2 * j) - m * 18;
-    dst[j] = make_double2(sm[m * kStagePitch + k], sm[m * kStagePitch + k + 1]);
-  }
+  stage_out(sm, aos, first, n);
 }
 
 inline unsigned nblocks(int64_t n, int thr) { return (unsigned)((n + thr - 1) / thr); }

@@ -17,6 +17,7 @@
 #include "lgf_df.cuh"
 #include "lgf_kernels.cuh"
 #include "lgf_reduce.cuh"
+#include "lgf_stage.cuh"
 
 namespace lgf {
 
@@ -148,30 +149,8 @@ __global__ void k_aos_to_soa(const double* __restrict__ aos, cx<T>* __restrict__
 
 // ---------------------------------------------------------------------------
 // Link loads and stores in the host layout (AoS, 18 doubles per link, 4 links
-// per site), staged through shared memory.  A CTA moves one contiguous chunk
-// of kStageMats links with 16-byte accesses; the staged rows have a pitch of
-// 19 doubles, which makes the per-thread 8-byte reads conflict-free.  The AoS
-// side may be host memory that the device reads or writes directly (pinned
-// memory over NVLink-C2C): every byte crosses once, coalesced.
+// per site), staged through shared memory (lgf_stage.cuh).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void stage_in(const double* __restrict__ aos, double* sm, int64_t first, int n) {
-  const double2* src = reinterpret_cast<const double2*>(aos + first * 18);
-  for (int j = threadIdx.x; j < n * 9; j += blockDim.x) {
-    const double2 v = src[j];  // doubles 2j and 2j+1 of the chunk: one link, entries k and k+1
-    const int m = (2 * j) / 18, k = (2 * j) - m * 18;
-    sm[m * kStagePitch + k] = v.x;
-    sm[m * kStagePitch + k + 1] = v.y;
-  }
-}
-
-__device__ __forceinline__ void stage_out(const double* sm, double* __restrict__ aos, int64_t first, int n) {
-  double2* dst = reinterpret_cast<double2*>(aos + first * 18);
-  for (int j = threadIdx.x; j < n * 9; j += blockDim.x) {
-    const int m = (2 * j) / 18, k = (2 * j) - m * 18;
-    dst[j] = make_double2(sm[m * kStagePitch + k], sm[m * kStagePitch + k + 1]);
-  }
-}
-
 // AoS links -> FP64 SoA (NC64 planes per direction, 0: none) and FP32 SoA
 // (NC32 planes, 0: none), one read of the input
 template <int NC64, int NC32>
@@ -205,13 +184,7 @@ __global__ void __launch_bounds__(kStageMats) k_store_aos(const cx<T>* __restric
     const int64_t i = first + threadIdx.x;
     const int64_t s = i >> 2;
     const int mu = (int)(i & 3);
-    const M3<T> m = load_m3<T, NC>(U + (int64_t)mu * NC * V, V, s);
-    double* d = sm + threadIdx.x * kStagePitch;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-      d[2 * c] = (double)m.e[c / 3][c % 3].re;
-      d[2 * c + 1] = (double)m.e[c / 3][c % 3].im;
-    }
+    stage_matrix(sm, load_m3<T, NC>(U + (int64_t)mu * NC * V, V, s));
   }
   __syncthreads();
   stage_out(sm, aos, first, n);
@@ -271,19 +244,19 @@ __global__ void __launch_bounds__(kStageMats) k_store_aos_df(const cx<float>* __
   stage_out(sm, aos, first, n);
 }
 
+// a gauge field (one matrix per site; row 3 rebuilt for NC = 6) -> [s][3][3]
+// doubles, staged: a thread writing its own 144-byte row left every store a
+// partial line, 48 GB/s into host memory (32^4: 2.9 ms); staged it runs at the
+// host link's rate
 template <class T, int NC>
-__global__ void k_soa_to_aos(const cx<T>* __restrict__ U, double* __restrict__ aos, int64_t V, int nmu) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nmu * V) return;
-  const int64_t s = i / nmu;
-  const int mu = (int)(i - s * nmu);
-  const M3<T> m = load_m3<T, NC>(U + (int64_t)mu * NC * V, V, s);
-  double* dst = aos + i * 18;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    dst[2 * c] = (double)m.e[c / 3][c % 3].re;
-    dst[2 * c + 1] = (double)m.e[c / 3][c % 3].im;
-  }
+__global__ void __launch_bounds__(kGaugeMats) k_store_gauge(const cx<T>* __restrict__ G, double* __restrict__ aos,
+                                                            int64_t V) {
+  __shared__ double sm[kGaugeMats * kStagePitch];
+  const int64_t first = (int64_t)blockIdx.x * kGaugeMats;
+  const int n = (int)(V - first < kGaugeMats ? V - first : kGaugeMats);
+  if ((int)threadIdx.x < n) stage_matrix(sm, load_m3<T, NC>(G, V, first + threadIdx.x));
+  __syncthreads();
+  stage_out(sm, aos, first, n);
 }
 
 // G(x) <- reunitarised g(x) G(x), in the storage precision
@@ -430,10 +403,9 @@ cudaError_t launch_store_aos(int prec, int nc, const void* U, double* aos, int64
   return cudaPeekAtLastError();
 }
 
-cudaError_t launch_soa_to_aos(int prec, int nc, const void* U, double* aos, int64_t V, int nmu, cudaStream_t s) {
-  LGF_DISPATCH(prec, nc,
-               (k_soa_to_aos<T, NC><<<blocks_for(nmu * V, 256), 256, 0, s>>>(static_cast<const cx<T>*>(U), aos, V,
-                                                                             nmu)));
+cudaError_t launch_store_gauge(int prec, int nc, const void* G, double* aos, int64_t V, cudaStream_t s) {
+  const unsigned nb = blocks_for(V, kGaugeMats);
+  LGF_DISPATCH(prec, nc, (k_store_gauge<T, NC><<<nb, kGaugeMats, 0, s>>>(static_cast<const cx<T>*>(G), aos, V)));
   return cudaPeekAtLastError();
 }
 

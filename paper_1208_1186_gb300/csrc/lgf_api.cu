@@ -1497,9 +1497,9 @@ int lgf_store_gauge(lgf_handle h, double* host_g) {
   if (h->mixed && h->cur == &h->e64 && h->df)
     LGF_LAUNCH(h, LGF_K_OTHER, launch_store_gauge_df(h->e64.g, h->eta, h->V, dst, h->stream));
   else if (h->mixed)
-    LGF_LAUNCH(h, LGF_K_OTHER, launch_soa_to_aos(4, h->e32.nc, h->G, dst, h->V, 1, h->stream));
+    LGF_LAUNCH(h, LGF_K_OTHER, launch_store_gauge(4, h->e32.nc, h->G, dst, h->V, h->stream));
   else
-    LGF_LAUNCH(h, LGF_K_OTHER, launch_soa_to_aos(8, h->e64.nc, h->G, dst, h->V, 1, h->stream));
+    LGF_LAUNCH(h, LGF_K_OTHER, launch_store_gauge(8, h->e64.nc, h->G, dst, h->V, h->stream));
   if (!direct)
     LGF_CUDA(h, cudaMemcpyAsync(host_g, h->staging, (size_t)h->V * 18 * sizeof(double), cudaMemcpyDeviceToHost,
                                 h->stream));
@@ -1727,7 +1727,7 @@ int lgf_probe(lgf_handle h, double* delta_packed, double* delta_tilde_packed, do
     LGF_CUDA(h, cudaStreamSynchronize(s));
   }
   if (g) {
-    LGF_LAUNCH(h, LGF_K_OTHER, launch_soa_to_aos(e.prec, e.nc, e.g, h->staging, V, 1, s));
+    LGF_LAUNCH(h, LGF_K_OTHER, launch_store_gauge(e.prec, e.nc, e.g, h->staging, V, s));
     LGF_CUDA(h, cudaMemcpyAsync(g, h->staging, (size_t)V * 18 * sizeof(double), cudaMemcpyDeviceToHost, s));
   }
   LGF_CUDA(h, cudaStreamSynchronize(s));
