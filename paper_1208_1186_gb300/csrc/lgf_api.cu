@@ -103,6 +103,8 @@ struct lgf_ctx {
   bool g_valid = false;       // G (with the tail's Gh, Gl and eta) describes the current links
   int tail_mode = 0;          // defect-correction tail when the FP32 phase reached 1e-8, with links in
                               // double-float (0) or FP64 (2); 1: plain FP64
+  void* Ufx = nullptr;        // plain FP64 handles: the links in fixed-point pairs while a queue runs
+  bool fx = false;            // ... the queue being built or captured runs on them
   bool defect = false;        // the FP64 engine runs the defect-correction tail
   bool df = false;            // ... on the double-float links in Udf (converted back at the end)
   void* Udf = nullptr;        // tail links in double-float: 36 V complex hi, then 36 V complex lo
@@ -136,7 +138,7 @@ struct lgf_ctx {
     unsigned long long cond = 0;
     long long launches = 0;  // kernels per iteration
   };
-  DevLoop loops[4];
+  DevLoop loops[5];
   cudaStream_t cap_stream = nullptr;  // capture stream of the loop bodies
   int last_n32 = 0, last_n64 = 0;  // split of the last lgf_fix
   std::string err;
@@ -505,9 +507,19 @@ int queue_iteration(lgf_handle h, Engine& e) {
     LGF_LAUNCH(h, LGF_K_UPDATE, launch_tail_update(e.U, f.g, h->geo, h->st, s));
     return LGF_OK;
   }
+  const bool exact = h->exp_order == 0;
+  if (h->fx) {
+    // plain FP64 on the links in fixed-point pairs; FP64 acceleration
+    LGF_LAUNCH(h, LGF_K_GRADIENT, launch_gradient_fx(e.nc, h->Ufx, e.D, h->partial, h->geo, h->st, 1, s));
+    int rc = queue_accelerate(h, e, h->st);
+    if (rc) return rc;
+    LGF_LAUNCH(h, LGF_K_BUILD_G, launch_build_g_fx(e.nc, e.D, e.g, h->V, 0.5 * h->alpha, exact, h->st, s));
+    LGF_LAUNCH(h, LGF_K_UPDATE, launch_update_fx(e.nc, h->Ufx, e.g, h->geo, h->st, s));
+    if (h->g64_track) LGF_LAUNCH(h, LGF_K_ACCUMULATE, launch_accumulate_fx(e.nc, h->G, e.g, h->V, h->st, s));
+    return LGF_OK;
+  }
   int rc = queue_gradient(h, e, 1);
   if (rc) return rc;
-  const bool exact = h->exp_order == 0;
   if (e.grep && !exact && pick_pipeline(h, e) == 3 && plane_xyinv_gstep_supported(e.prec, h->L[0])) {
     // forward x-y, z-t, then the inverse x-y fused with G <- g G
     const int* L = h->L;
@@ -536,8 +548,10 @@ int queue_iteration(lgf_handle h, Engine& e) {
 
 // Device-side loops.  Kind 0: an iteration of the FP32 engine (or of a plain
 // FP32/FP64 handle's engine); 1: the double-float defect tail; 2: the FP64
-// defect tail; 3: the plain FP64 iteration of a mixed handle's tail.
+// defect tail; 3: the plain FP64 iteration of a mixed handle's tail; 4: the
+// plain FP64 iteration on fixed-point pairs.
 int loop_kind(lgf_handle h, const Engine& e) {
+  if (h->fx) return 4;
   if (&e == &h->e32 || !h->mixed) return 0;
   if (h->defect) return h->df ? 1 : 2;
   return 3;
@@ -601,6 +615,18 @@ int build_loop(lgf_handle h, Engine& e, lgf_ctx::DevLoop& l) {
   return LGF_OK;
 }
 
+// The links in fixed-point pairs from the FP64 links, and back, around an
+// iteration queue that runs on them (h->fx).
+int queue_fx_load(lgf_handle h, Engine& e) {
+  if (h->fx) LGF_LAUNCH(h, LGF_K_OTHER, launch_fx_load(e.nc, e.U, h->Ufx, h->V, h->st, h->stream));
+  return LGF_OK;
+}
+
+int queue_fx_store(lgf_handle h, Engine& e) {
+  if (h->fx) LGF_LAUNCH(h, LGF_K_OTHER, launch_fx_store(e.nc, h->Ufx, e.U, h->V, h->st, h->stream));
+  return LGF_OK;
+}
+
 // Run engine e until theta < tol, max_iter updates, or (if stall_check) theta
 // below 1e-6 has not halved within 8 updates (the stop rule is applied on the
 // device, lgf_reduce.cuh).  Without profiling the whole queue is one graph
@@ -608,8 +634,11 @@ int build_loop(lgf_handle h, Engine& e, lgf_ctx::DevLoop& l) {
 // between launches, the host queues iterations and checks between batches of
 // them.  Both run the same kernels and stop at the same update.  Returns
 // LGF_OK / error and the number of updates through *done_iters.
-int run_fix(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
-            int* done_iters, bool* converged) {
+// With h->fx the queue runs on the links in fixed-point pairs, formed from
+// the FP64 links before it and written back to them after it; *unfit reports
+// links that do not fit the pairs (nothing was done then).
+int run_queue(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
+              int* done_iters, bool* converged, bool* unfit) {
   *converged = false;
   if (!h->profiling && kDeviceLoops) {
     lgf_ctx::DevLoop& l = h->loops[loop_kind(h, e)];
@@ -618,11 +647,17 @@ int run_fix(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
       if (rc) return rc;
     }
     int rc = reset_state(h, tol, max_iter, true, stall_check, true, l.cond);
+    if (!rc) rc = queue_fx_load(h, e);
     if (rc) return rc;
     LGF_CUDA(h, cudaGraphLaunch(l.exec, h->stream));
-    rc = sync_state(h);
+    rc = queue_fx_store(h, e);
+    if (!rc) rc = sync_state(h);
     if (rc) return rc;
     const DevState& s = *h->st_host;
+    if (s.unfit) {
+      *unfit = true;
+      return LGF_OK;
+    }
     h->launches += (long long)(s.iters + 1) * l.launches;
     if (s.nonfinite) return fail(h, LGF_ERR_NONFINITE, "F or theta is not finite (non-SU(3) or NaN input links?)");
     *done_iters = s.iters;
@@ -631,6 +666,7 @@ int run_fix(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
     return LGF_OK;
   }
   int rc = reset_state(h, tol, max_iter, true, stall_check);
+  if (!rc) rc = queue_fx_load(h, e);
   if (rc) return rc;
   long long queued = 0;
   // queue length: 8 iterations first, then as many as the measured contraction
@@ -651,6 +687,10 @@ int run_fix(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
     rc = sync_state(h);
     if (rc) return rc;
     const DevState& s = *h->st_host;
+    if (s.unfit) {
+      *unfit = true;
+      return LGF_OK;
+    }
     if (s.nonfinite) return fail(h, LGF_ERR_NONFINITE, "F or theta is not finite (non-SU(3) or NaN input links?)");
     if (s.done || queued >= (long long)max_iter + 1) break;
     // predict the iterations still needed from the last interval
@@ -667,11 +707,28 @@ int run_fix(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
     prev_theta = s.theta;
     prev_iters = s.iters;
   }
+  rc = queue_fx_store(h, e);
+  if (!rc && h->fx) rc = sync_state(h);
+  if (rc) return rc;
   const DevState& s = *h->st_host;
   *done_iters = s.iters;
   h->hist_n = s.iters + 1 < h->hist_cap ? s.iters + 1 : h->hist_cap;
   *converged = s.theta < tol;
   return LGF_OK;
+}
+
+// run_queue on the fixed-point pairs of a plain FP64 handle where its links
+// fit them, else on the engine's own links.
+int run_fix(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
+            int* done_iters, bool* converged) {
+  bool unfit = false;
+  if (h->Ufx) {
+    h->fx = true;
+    const int rc = run_queue(h, e, tol, max_iter, stall_check, done_iters, converged, &unfit);
+    h->fx = false;
+    if (rc || !unfit) return rc;
+  }
+  return run_queue(h, e, tol, max_iter, stall_check, done_iters, converged, &unfit);
 }
 
 }  // namespace
@@ -989,25 +1046,62 @@ int read_members(lgf_batch b, const std::vector<int>& members) {
   return LGF_OK;
 }
 
+// queue_fx_load or queue_fx_store of the listed members on the main stream
+int queue_fx_members(lgf_batch b, const std::vector<int>& members, int (*queue)(lgf_handle, Engine&)) {
+  for (int i : members) {
+    lgf_handle h = b->h[i];
+    cudaStream_t saved = h->stream;
+    h->stream = b->main;
+    const int rc = queue(h, *h->cur);
+    h->stream = saved;
+    if (rc) return bfail(b, rc, h->err);
+  }
+  return LGF_OK;
+}
+
 // Run the listed members until each has stopped (theta < tol, its update
 // budget, or -- with stall_check -- theta below 1e-6 no longer halving within
 // 8 updates): one launch of the batch graph, every member looping on the
 // device until its own stop decision.
+// Plain FP64 members run on their links in fixed-point pairs (allow_fx);
+// those whose links do not fit run again on their FP64 links.
 int run_members(lgf_batch b, const std::vector<int>& members, const std::vector<double>& tol,
-                const std::vector<int>& max_iter, const std::vector<char>& stall_check) {
+                const std::vector<int>& max_iter, const std::vector<char>& stall_check, bool allow_fx = true) {
   if (members.empty()) return LGF_OK;
+  for (int i : members) b->h[i]->fx = allow_fx && b->h[i]->Ufx;
+  auto leave_fx = [&](int rc) {
+    for (int i : members) b->h[i]->fx = false;
+    return rc;
+  };
   std::vector<unsigned long long> conds;
   int rc = capture(b, members, conds);
-  if (rc) return rc;
-  rc = reset_members(b, members, tol, max_iter, stall_check, conds);
-  if (rc) return rc;
-  LGF_BCUDA(b, cudaGraphLaunch(b->exec, b->main));
-  rc = read_members(b, members);
-  if (rc) return rc;
+  if (!rc) rc = reset_members(b, members, tol, max_iter, stall_check, conds);
+  if (!rc) rc = queue_fx_members(b, members, queue_fx_load);
+  if (!rc && cudaGraphLaunch(b->exec, b->main) != cudaSuccess)
+    rc = bfail(b, LGF_ERR_CUDA, "batch graph: launch failed");
+  if (!rc) rc = queue_fx_members(b, members, queue_fx_store);
+  if (!rc) rc = read_members(b, members);
+  if (leave_fx(rc)) return rc;
+  std::vector<int> again, cap2;
+  std::vector<double> tol2;
+  std::vector<char> stall2;
+  for (size_t m = 0; m < members.size(); ++m) {
+    if (!b->h[members[m]]->st_host->unfit) continue;
+    again.push_back(members[m]);
+    tol2.push_back(tol[m]);
+    cap2.push_back(max_iter[m]);
+    stall2.push_back(stall_check[m]);
+  }
+  const std::vector<long long> per_iter = b->exec_launches;
+  if (!again.empty()) {
+    rc = run_members(b, again, tol2, cap2, stall2, false);
+    if (rc) return rc;
+  }
   for (size_t m = 0; m < members.size(); ++m) {
     lgf_handle h = b->h[members[m]];
+    if (std::find(again.begin(), again.end(), members[m]) != again.end()) continue;
     const DevState& s = *h->st_host;
-    h->launches += (long long)(s.iters + 1) * b->exec_launches[m];
+    h->launches += (long long)(s.iters + 1) * per_iter[m];
     if (s.nonfinite)
       return bfail(b, LGF_ERR_NONFINITE, "member " + std::to_string(members[m]) + ": F or theta is not finite");
     h->hist_n = s.iters + 1 < h->hist_cap ? s.iters + 1 : h->hist_cap;
@@ -1268,6 +1362,8 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
   }
   if (rc) return bail(rc);
   h->cur = h->mixed ? &h->e32 : &h->e64;
+  // without it (no memory left) the handle iterates on its FP64 links
+  if (!h->mixed) h->Ufx = dev_alloc(h, (size_t)4 * h->e64.nc * V * 16);
   if (h->mixed) {
     h->G = dev_alloc(h, (size_t)h->e32.nc * V * h->e32.cbytes());
     h->Uorig = static_cast<double*>(dev_alloc(h, (size_t)4 * 9 * V * 16));
@@ -1510,13 +1606,19 @@ int lgf_store_gauge(lgf_handle h, double* host_g) {
 int lgf_iterate(lgf_handle h, int n) {
   if (!h || n < 0) return LGF_ERR_ARG;
   if (!h->loaded) return fail(h, LGF_ERR_ARG, "no links loaded");
-  int rc = reset_state(h, -1.0, n, false);
-  if (rc) return rc;
-  for (int i = 0; i < n; ++i) {
-    rc = queue_iteration(h, *h->cur);
-    if (rc) return rc;
+  // first on the fixed-point pairs of a plain FP64 handle, then, if its links
+  // do not fit them (nothing was done), on the engine's own links
+  int rc = LGF_OK;
+  for (int pass = h->Ufx ? 0 : 1; pass < 2 && !rc; ++pass) {
+    h->fx = pass == 0;
+    rc = reset_state(h, -1.0, n, false);
+    if (!rc) rc = queue_fx_load(h, *h->cur);
+    for (int i = 0; i < n && !rc; ++i) rc = queue_iteration(h, *h->cur);
+    if (!rc) rc = queue_fx_store(h, *h->cur);
+    h->fx = false;
+    if (!rc) rc = sync_state(h);
+    if (!rc && !h->st_host->unfit) break;
   }
-  rc = sync_state(h);
   if (rc) return rc;
   if (h->st_host->nonfinite) return fail(h, LGF_ERR_NONFINITE, "F or theta is not finite");
   h->total_updates += h->st_host->iters;

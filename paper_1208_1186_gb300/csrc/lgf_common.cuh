@@ -392,6 +392,7 @@ struct DevState {
   int done;          // 1: no further update is applied
   int iters;         // updates applied since the last reset
   int nonfinite;     // F or theta was NaN/Inf
+  int unfit;         // the links do not fit the fixed-point pairs (k_links_fx.cu); no update was applied
   int max_iter;      // stop once iters reaches this (fix mode)
   double tol;        // stop once theta < tol (fix mode; < 0 disables)
   int hist_cap;

@@ -1,0 +1,138 @@
+// Fixed-point pairs: the working form of the links and of g in the plain FP64
+// iteration.
+//
+// FP64 runs at 1/62 of the FP32 rate on this GPU (about 2 multiply-adds per
+// clock and SM), so the 864 multiply-adds of the link update alone took half of
+// the FP64 iteration.  Every number the products multiply is an entry of a
+// unitary matrix, at most 1 in magnitude, so it needs no exponent:
+//
+//   x = (h + l) 2^-30,  h a 32-bit integer, l an FP32 number with |l| <= 1/2,
+//
+// a resolution of 2^-55 (FP64 resolves 2^-53 of a number near 1).  A product
+// is
+//
+//   x y 2^60 = h_x h_y + (h_x l_y + l_x h_y) + l_x l_y:
+//
+// the first term exact in a 64-bit integer accumulator (one 32 x 32 + 64
+// multiply-add; 32 a clock and SM), the second in an FP32 accumulator (two
+// FMAs; the rounding of a term below 2^29 is 2^5, i.e. 2^-55 of the result),
+// the third, at most 1/4, dropped.  A dot product of six terms is off by about
+// 2^-54, where six FP64 roundings leave about 2^-53.
+//
+// Range: |h| < 2^31 holds |x| < 2; rows of norm at most 1 + 2^-7 times unitary
+// matrices keep every entry below 1.75 and every accumulator below 2^62.
+#pragma once
+
+#include "lgf_common.cuh"
+
+namespace lgf {
+
+// one complex number
+struct alignas(16) fx {
+  int hr;
+  float lr;
+  int hi;
+  float li;
+};
+
+__device__ __forceinline__ fx fx_ldg(const fx* p) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  return {v.x, __int_as_float(v.y), v.z, __int_as_float(v.w)};
+}
+
+__device__ __forceinline__ fx fx_neg(fx a) { return {-a.hr, -a.lr, -a.hi, -a.li}; }
+
+// a real operand with its integer part also in FP32
+struct fxr {
+  int h;
+  float l, f;
+};
+
+__device__ __forceinline__ fxr fx_re(const fx& a) { return {a.hr, a.lr, (float)a.hr}; }
+__device__ __forceinline__ fxr fx_im(const fx& a) { return {a.hi, a.li, (float)a.hi}; }
+__device__ __forceinline__ fxr fx_neg(fxr a) { return {-a.h, -a.l, -a.f}; }
+
+struct fxacc {
+  long long h;
+  float l;
+};
+
+// a += x y
+__device__ __forceinline__ void fx_mac(fxacc& a, const fxr& x, const fxr& y) {
+  a.h += (long long)x.h * (long long)y.h;
+  a.l = __fmaf_rn(x.f, y.l, __fmaf_rn(x.l, y.f, a.l));
+}
+
+// an accumulated product sum, in units of 2^-60, as h and l
+__device__ __forceinline__ void fx_round(const fxacc& a, int& h, float& l) {
+  h = (int)((a.h + (1ll << 29)) >> 30);
+  const int rem = (int)((unsigned)a.h - ((unsigned)h << 30));  // |rem| <= 2^29
+  const float t = __fmul_rn(__fadd_rn((float)rem, a.l), 0x1p-30f);
+  const float k = __fadd_rn(t, 12582912.f);  // 1.5 2^23: t rounded to an integer in the low bits
+  h += __float_as_int(k) - 0x4B400000;
+  l = __fsub_rn(t, __fsub_rn(k, 12582912.f));
+}
+
+__device__ __forceinline__ fx fx_round(const fxacc& re, const fxacc& im) {
+  fx r;
+  fx_round(re, r.hr, r.lr);
+  fx_round(im, r.hi, r.li);
+  return r;
+}
+
+// entry j of row 3 of an SU(3) matrix from rows 1 and 2: conj(r1 x r2)
+__device__ __forceinline__ fx fx_row3(const fx* r1, const fx* r2, int j) {
+  const int k = (j + 1) % 3, l = (j + 2) % 3;
+  const fxr ukr = fx_re(r1[k]), uki = fx_im(r1[k]), ulr = fx_re(r1[l]), uli = fx_im(r1[l]);
+  const fxr vkr = fx_re(r2[k]), vki = fx_im(r2[k]), vlr = fx_re(r2[l]), vli = fx_im(r2[l]);
+  fxacc re = {0, 0.f}, im = {0, 0.f};
+  fx_mac(re, ukr, vlr);
+  fx_mac(re, fx_neg(uki), vli);
+  fx_mac(re, fx_neg(ulr), vkr);
+  fx_mac(re, uli, vki);
+  fx_mac(im, fx_neg(ukr), vli);
+  fx_mac(im, fx_neg(uki), vlr);
+  fx_mac(im, ulr, vki);
+  fx_mac(im, uli, vkr);
+  return fx_round(re, im);
+}
+
+// FP64 -> (h, l) by bit manipulation (FP64 arithmetic and conversions run at
+// the FP64 rate); false for |x| >= 2 and for non-finite x
+__device__ __forceinline__ bool fx_from_double(double x, int& h, float& l) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ffull) - 1023;
+  const unsigned long long m = ((b << 11) | (1ull << 63));  // |x| = m 2^(e - 63)
+  const int sh = 1 - e;                                      // |x| = (m >> sh) 2^-62
+  long long f = sh < 64 ? (long long)(m >> (sh & 63)) : 0;
+  if ((long long)b < 0) f = -f;
+  h = (int)((f + (1ll << 31)) >> 32);
+  l = __fmul_rn((float)(int)(unsigned)f, 0x1p-32f);
+  return e <= 0;
+}
+
+// f 2^-kScale as the nearest FP64 number, by bit manipulation
+template <int kScale>
+__device__ __forceinline__ double fx_scaled_to_double(long long f) {
+  unsigned long long u = f < 0 ? 0ull - (unsigned long long)f : (unsigned long long)f;
+  if (u == 0) return 0.0;
+  const int n = __clzll((long long)u);
+  u <<= n;  // the leading bit at 63
+  unsigned long long v = u >> 11;
+  const unsigned r = (unsigned)u & 0x7ffu;
+  v += (r > 0x400u || (r == 0x400u && (v & 1))) ? 1ull : 0ull;
+  // the leading bit of v adds one to the exponent field (and a carry another)
+  v += (unsigned long long)(1023 + 63 - n - kScale - 1) << 52;
+  return __longlong_as_double((long long)(v | (f < 0 ? 1ull << 63 : 0ull)));
+}
+
+__device__ __forceinline__ double fx_to_double(int h, float l) {
+  return fx_scaled_to_double<62>(((long long)h << 32) + (long long)__float2int_rn(__fmul_rn(l, 0x1p32f * 0.5f)) * 2);
+}
+
+// a sum of (h, l) pairs, in units of 2^-30 and at most 2^34 of them, as FP64
+__device__ __forceinline__ double fx_sum_to_double(const fxacc& a) {
+  return fx_scaled_to_double<58>((a.h << 28) + __float2int_rn(__fmul_rn(a.l, 0x1p28f)));
+}
+
+}  // namespace lgf

@@ -75,6 +75,17 @@ cudaError_t launch_build_g(int prec, int nc, const void* D, void* g, int64_t V, 
                            bool reunit_fp64, bool exact, const DevState* st, cudaStream_t s);
 cudaError_t launch_update(int prec, int nc, void* U, const void* g, const Geom& geo,
                           const DevState* st, cudaStream_t s);
+// the plain FP64 iteration on links in fixed-point pairs (k_links_fx.cu; lgf_fx.cuh): Ufx and g hold
+// nc planes of 16-byte complex pairs per matrix.  launch_fx_load stops the queue with st->unfit if the
+// links do not fit the pairs' range; launch_fx_store leaves U64 alone then, or if no update was applied
+cudaError_t launch_fx_load(int nc, const void* U64, void* Ufx, int64_t V, DevState* st, cudaStream_t s);
+cudaError_t launch_fx_store(int nc, const void* Ufx, void* U64, int64_t V, const DevState* st, cudaStream_t s);
+cudaError_t launch_gradient_fx(int nc, const void* Ufx, void* D, double2* partial, const Geom& geo, DevState* st,
+                               int mode, cudaStream_t s);
+cudaError_t launch_build_g_fx(int nc, const void* D, void* g, int64_t V, double half_alpha, bool exact, DevState* st,
+                              cudaStream_t s);
+cudaError_t launch_update_fx(int nc, void* Ufx, const void* g, const Geom& geo, const DevState* st, cudaStream_t s);
+cudaError_t launch_accumulate_fx(int nc, void* G, const void* g, int64_t V, const DevState* st, cudaStream_t s);
 // host [s][mu][3][3] complex128 layout (on the device) <-> SoA storage
 // (nmu matrices per site: 4 for links, 1 for a gauge field)
 cudaError_t launch_aos_to_soa(int prec, int nc, const double* aos, void* U, int64_t V, int nmu, cudaStream_t s);
@@ -210,6 +221,6 @@ constexpr int kGradThreads = 256;  // k_gradient block size
 constexpr int kGrepThreads = 256;  // k_gradient_grep block size
 inline int gradient_blocks(int64_t V) { return (int)((V + kGradThreads - 1) / kGradThreads); }
 // capacity of the block-partials buffer: enough for the smallest block size
-inline int64_t partial_capacity(int64_t V) { return (V + 63) / 64 + 1; }
+inline int64_t partial_capacity(int64_t V) { return (V + 31) / 32 + 1; }
 
 }  // namespace lgf
