@@ -5,9 +5,9 @@
 //
 // Network: three 3^4-tap periodic convolutions, 48 -> 32 -> 32 -> 8 channels,
 // ReLU after the first two; BF16 weights and activations, FP32 accumulation
-// on the tensor cores (the forward and backward-data convolutions as
-// tcgen05 implicit GEMMs, the weight gradient on warp-level 16x16x16 BF16
-// tiles), FP32 master weights and Adam moments.  Training signal: the loss is -F(U^{g0}) (the
+// on the tensor cores (the forward and backward-data convolutions and the
+// weight gradients as tcgen05 implicit GEMMs), FP32 master weights and Adam
+// moments.  Training signal: the loss is -F(U^{g0}) (the
 // method's own functional), whose derivative along left translations of
 // g0(x) is the projection of the transformed links' gradient Delta'(x) onto
 // the su(3) generators; Delta' comes from the gauge-representation gradient
@@ -16,7 +16,6 @@
 // Layouts: activations [site][channel] (BF16, channels fastest), weights
 // [tap][in][out] with tap = ((dt*3 + dz)*3 + dy)*3 + dx, offsets d - 1.
 #include <cuda_bf16.h>
-#include <mma.h>
 
 #include "lgf_kernels.cuh"
 
@@ -24,7 +23,6 @@ namespace lgf {
 namespace warm {
 
 using bf16 = __nv_bfloat16;
-namespace wm = nvcuda::wmma;
 
 constexpr int kFeat = 48;  // 32 link coefficients + 6 plaquettes + 10 zeros
 constexpr int kHid = 32;
@@ -190,23 +188,6 @@ __global__ void __launch_bounds__(128) k_signal(const cx<float>* __restrict__ D,
   bf16* out = gc + (size_t)s * kOutPad;
 #pragma unroll
   for (int a = 0; a < 16; a += 2) *reinterpret_cast<__nv_bfloat162*>(out + a) = __floats2bfloat162_rn(coef * p[a], coef * p[a + 1]);
-}
-
-// ---------------------------------------------------------------------------
-// convolutions on the tensor cores
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ int wrapc(int c, int d, int L) {
-  int v = c + d;
-  v = v < 0 ? v + L : v;
-  return v >= L ? v - L : v;
-}
-
-// neighbour of site s (coordinates c) at tap offset (sign * (d - 1))
-__device__ __forceinline__ int tap_site(const Geom& geo, const int c[4], int tap, int sign) {
-  const int d0 = sign * (tap % 3 - 1), d1 = sign * ((tap / 3) % 3 - 1);
-  const int d2 = sign * ((tap / 9) % 3 - 1), d3 = sign * (tap / 27 - 1);
-  return wrapc(c[0], d0, geo.L[0]) +
-         geo.L[0] * (wrapc(c[1], d1, geo.L[1]) + geo.L[1] * (wrapc(c[2], d2, geo.L[2]) + geo.L[2] * wrapc(c[3], d3, geo.L[3])));
 }
 
 // ---------------------------------------------------------------------------
@@ -613,74 +594,254 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const bf16* __restrict__
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
 }
 
-// gW[tap, i, o] += sum_s x[s + off(tap), i] gy[s, o]: block (chunk group,
-// tap); each warp accumulates 16-site chunks on the tensor cores and adds its
-// tile to gW with FP32 atomics (so the sum order, and its last bits, vary).
-template <int CI, int CO>
-__global__ void __launch_bounds__(128) k_conv_bwd_weight(const bf16* __restrict__ x, const bf16* __restrict__ gy,
-                                                         float* __restrict__ gW, const Geom geo, int chunks_per_warp) {
-  __shared__ __align__(32) bf16 sX[4][16 * CI];
-  __shared__ __align__(32) float sC[4][CI * CO];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int V = (int)geo.V;
-  const int tap = blockIdx.y;
-  wm::fragment<wm::accumulator, 16, 16, 16, float> acc[CI / 16][CO / 16];
-#pragma unroll
-  for (int m = 0; m < CI / 16; ++m)
-#pragma unroll
-    for (int n = 0; n < CO / 16; ++n) wm::fill_fragment(acc[m][n], 0.0f);
-  const int first = (blockIdx.x * 4 + warp) * chunks_per_warp;
-  for (int ch = 0; ch < chunks_per_warp; ++ch) {
-    const int s0 = (first + ch) * 16;
-    if (s0 >= V) break;
-    // stage the 16 neighbour rows of x (CI channels each)
-    for (int e = lane; e < 16 * (CI / 8); e += 32) {
-      const int r = e / (CI / 8), q = e % (CI / 8);
-      int c[4];
-      site_coords_i(geo.L, s0 + r, c);
-      const int nb = tap_site(geo, c, tap, +1);
-      *reinterpret_cast<uint4*>(&sX[warp][r * CI + q * 8]) =
-          *reinterpret_cast<const uint4*>(x + (size_t)nb * CI + q * 8);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < CI / 16; ++m) {
-      // A[m = i][k = site] = sX[site][i]: column-major, leading dimension CI
-      wm::fragment<wm::matrix_a, 16, 16, 16, bf16, wm::col_major> am;
-      wm::load_matrix_sync(am, &sX[warp][m * 16], CI);
-#pragma unroll
-      for (int n = 0; n < CO / 16; ++n) {
-        wm::fragment<wm::matrix_b, 16, 16, 16, bf16, wm::row_major> bm;
-        wm::load_matrix_sync(bm, gy + (size_t)s0 * CO + n * 16, CO);
-        wm::mma_sync(acc[m][n], am, bm, acc[m][n]);
-      }
-    }
-    __syncwarp();
-  }
-#pragma unroll
-  for (int m = 0; m < CI / 16; ++m)
-#pragma unroll
-    for (int n = 0; n < CO / 16; ++n)
-      wm::store_matrix_sync(&sC[warp][(m * 16) * CO + n * 16], acc[m][n], CO, wm::mem_row_major);
-  __syncwarp();
-  float* dst = gW + (size_t)tap * CI * CO;
-  for (int e = lane; e < CI * CO; e += 32) atomicAdd(dst + e, sC[warp][e]);
+// ---------------------------------------------------------------------------
+// weight gradients on the tensor cores (tcgen05):
+//   gW[tap, i, o] += sum_s x[s + off(tap), i] gy[s, o],
+// a GEMM whose K is the sites.  Rows run over the same lattice with a periodic
+// x and y halo as k_conv_tc's; row P of a (z, t) plane holds the x site of its
+// position, and with gy zero on the halo every tap (dx, dy) of a (dz, dt) is
+//   sum_P x_(dz, dt)[P] gy[P - dx - dy (Lx + 2)].
+// So the nine shifts go to gy: M stacks the shifted copies of gy (9 x 32
+// channels in three tiles of 128; 9 x 8 in one for the last layer, of whose 16
+// channels 8 are used), N stacks the channels of the three dz windows of x
+// (144 or 96), and dt is the grid's y.  All of a CTA's D, M x N up to
+// 3 x 128 x 144, stays in tensor memory (432 of 512 columns) while the CTA
+// walks its share of the rows, 64 a stage; it ends in one FP32 addition per
+// element and CTA to gW (coalesced, so a warp's 32 go to L2 as one).
+//
+// N is that wide because the operands come from shared memory: an MMA of N =
+// 144 reads 8.6 KB for 590 kFLOP, against 5 KB for 131 kFLOP at N = 32.
+//
+// Both operands have the sites along K and the channels contiguous in memory:
+// MN-major, no swizzle, in the chunk-major layout of k_conv_tc (16-byte chunk c
+// of row r at c ROWS 16 + r 16: 128 bytes to the next 8 rows of K, ROWS x 16 to
+// the next 8 channels).  The third M tile reads 12 chunks past the ninth copy,
+// inside the stage's x windows; those rows of D are dropped.
+//
+// 16^4, us under ncu: layer 1 255 -> 42, layer 2 171 -> 37, layer 3 130 -> 21, from
+// warp-level mma tiles with 16-site chunks gathered per tap and 63 million FP32
+// atomics in layer 1 alone.
+// ---------------------------------------------------------------------------
+constexpr int kWgRows = 64;
+constexpr int kWgStages = 4;
+constexpr int kWgLag = 2;  // stages a producer keeps in flight before it hands one over
+constexpr uint32_t kWgChunk = kWgRows * 16;
+
+// CI channels of x, GC 16-byte chunks of gy used per shift
+template <int CI, int GC>
+struct WgShape {
+  static constexpr int kAChunks = 9 * GC, kBChunks = 3 * (CI / 8);
+  static constexpr int kMTiles = (kAChunks + 15) / 16;
+  static constexpr int kN = 3 * CI;
+  static constexpr int kCols = kMTiles * kN <= 128 ? 128 : 512;  // tensor memory columns (a power of two)
+  static constexpr uint32_t kABytes = kAChunks * kWgChunk;
+  static constexpr uint32_t kStage = (kAChunks + kBChunks) * kWgChunk;
+  static constexpr int kSmem = kWgStages * (int)kStage;
+  static_assert(kMTiles * 16 <= kAChunks + kBChunks, "the last M tile stays inside the stage");
+  static_assert(kN % 16 == 0 && kN <= 256 && kMTiles * kN <= 512, "one accumulator per M tile");
+  static_assert(kSmem <= 227 * 1024, "the stages fit one CTA's shared memory");
+};
+
+// 16 bytes global -> shared, zeros if !ok (src is then not read)
+__device__ __forceinline__ void cp_async16_or_zero(uint32_t sdst, const void* gsrc, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"(sdst), "l"(gsrc), "r"(ok ? 16 : 0) : "memory");
 }
 
-// gb[o] += sum_s gy[s, o]
-template <int CO>
-__global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ gy, float* __restrict__ gb, int V) {
-  __shared__ float part[256 / CO][CO];
-  const int o = threadIdx.x % CO, r = threadIdx.x / CO;
-  constexpr int R = 256 / CO;
-  float acc = 0.f;
-  for (int s = blockIdx.x * R + r; s < V; s += gridDim.x * R) acc += __bfloat162float(gy[(size_t)s * CO + o]);
-  part[r][o] = acc;
+// gy rows have LG channels; gW rows LO
+template <int CI, int GC, int LG, int LO>
+__global__ void __launch_bounds__(kTcThreads) k_wgrad_tc(const bf16* __restrict__ x, const bf16* __restrict__ gy,
+                                                        float* __restrict__ gW, const Geom geo, int nchunks,
+                                                        int* __restrict__ err) {
+  using S = WgShape<CI, GC>;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t full[kWgStages];   // a stage has landed (128 producer arrivals)
+  __shared__ __align__(8) uint64_t empty[kWgStages];  // the MMAs reading a stage have completed
+  __shared__ __align__(8) uint64_t done_bar;          // all MMAs have completed
+  __shared__ uint32_t tmem_slot;
+  __shared__ int stop, last_issued;
+  const int t = threadIdx.x, w = t >> 5;
+  const bool producer = t < 128, issuer = t == 128;
+  const int Lx = geo.L[0], Ly = geo.L[1], Lz = geo.L[2], Lt = geo.L[3];
+  const int LXP = Lx + 2, PLANE = LXP * (Ly + 2), PR = PLANE * Lz * Lt;
+  const int first = (int)((int64_t)nchunks * blockIdx.x / gridDim.x);
+  const int n = (int)((int64_t)nchunks * (blockIdx.x + 1) / gridDim.x) - first;
+  const uint32_t sbase = smem_u32(smem_raw);
+  if (t == 0) {
+    for (int k = 0; k < kWgStages; ++k) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;" ::"r"(smem_u32(&full[k])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[k])) : "memory");
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&done_bar)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    stop = 0;
+    last_issued = -1;
+  }
+  if (w == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(S::kCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (r == 0) {
-    float t = 0.f;
-    for (int k = 0; k < R; ++k) t += part[k][o];
-    atomicAdd(gb + o, t);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+  const unsigned stage_polls = (unsigned)err[1];
+  auto fail = [&]() {
+    atomicExch(err, 1);
+    *(volatile int*)&stop = 1;
+  };
+
+  if (producer) {
+    // thread = (row of the stage, half); the halves share a row's copies about
+    // equally: with four chunks per shift, shifts 0-6 against 7, 8 and the
+    // x windows
+    constexpr int kSplit = GC == 4 ? 7 : 9;
+    const int r = t & (kWgRows - 1), half = t / kWgRows;
+    const int dt = (int)blockIdx.y - 1;
+    auto fill = [&](int i) {
+      const uint32_t row = sbase + (i % kWgStages) * S::kStage + r * 16;
+      const int P = (first + i) * kWgRows + r;
+      const bool in = P < PR;
+      const int l = in ? P / PLANE : 0, q = in ? P - l * PLANE : 0;
+      const int yp = q / LXP, xp = q - yp * LXP;
+#pragma unroll
+      for (int j = 0; j < 9; ++j) {
+        if ((j < kSplit) != (half == 0)) continue;
+        const int xq = xp - (j % 3 - 1), yq = yp - (j / 3 - 1);
+        const bool ok = in && xq >= 1 && xq <= Lx && yq >= 1 && yq <= Ly;
+        const bf16* p = gy + (ok ? (size_t)((xq - 1) + Lx * ((yq - 1) + Ly * l)) * LG : 0);
+#pragma unroll
+        for (int c = 0; c < GC; ++c) cp_async16_or_zero(row + (j * GC + c) * kWgChunk, p + c * 8, ok);
+      }
+      if (half == 1) {
+        const int xs = xp == 0 ? Lx - 1 : (xp == Lx + 1 ? 0 : xp - 1);
+        const int ys = yp == 0 ? Ly - 1 : (yp == Ly + 1 ? 0 : yp - 1);
+        const int z = l % Lz, tt = wrap_add(l / Lz, dt, Lt);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const bf16* p = x + (size_t)(xs + Lx * (ys + Ly * (wrap_add(z, k - 1, Lz) + Lz * tt))) * CI;
+#pragma unroll
+          for (int c = 0; c < CI / 8; ++c)
+            cp_async16_or_zero(row + S::kABytes + (k * (CI / 8) + c) * kWgChunk, p + c * 8, in);
+        }
+      }
+    };
+    auto arrive = [&](int i) {  // this thread's copies of stage i have landed
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[i % kWgStages])) : "memory");
+    };
+    bool ok = true;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      if (i >= kWgStages && !mbar_wait_or_stop(&empty[i % kWgStages], (uint32_t)(((i - kWgStages) / kWgStages) & 1),
+                                               stage_polls, &stop)) {
+        fail();
+        ok = false;
+        break;
+      }
+      fill(i);
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      if (i >= kWgLag) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(kWgLag) : "memory");
+        arrive(i - kWgLag);
+      }
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if (ok)
+      for (int i = n > kWgLag ? n - kWgLag : 0; i < n; ++i) arrive(i);
+  } else if (issuer) {
+    constexpr uint32_t idesc = tc_idesc<S::kN>() | (1u << 15) | (1u << 16);  // A and B MN-major
+    int issued = -1;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      if (!mbar_wait_or_stop(&full[i % kWgStages], (uint32_t)((i / kWgStages) & 1), stage_polls, &stop)) {
+        fail();
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t st = sbase + (i % kWgStages) * S::kStage;
+      const uint64_t ad = tc_desc(st, 128, kWgChunk), bd = tc_desc(st + S::kABytes, 128, kWgChunk);
+#pragma unroll
+      for (int k = 0; k < kWgRows / 16; ++k)
+#pragma unroll
+        for (int m = 0; m < S::kMTiles; ++m)
+          tc_mma(tmem + m * S::kN, ad + ((m * 16 * kWgChunk + k * 256) >> 4), bd + (k * 256 >> 4), idesc,
+                 (i > 0 || k > 0) ? 1u : 0u);
+      tc_commit(&empty[i % kWgStages]);
+      issued = i;
+    }
+    if (issued >= 0) {
+      tc_commit(&done_bar);
+      if (!mbar_wait(&done_bar, 0u, kTcWaitLimit)) fail();
+    }
+    last_issued = issued;
+  }
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (producer && !stop && last_issued == n - 1) {
+    float* out = gW + (size_t)blockIdx.y * 27 * CI * LO;
+#pragma unroll 1
+    for (int m = 0; m < S::kMTiles; ++m) {
+      const int row = m * 128 + t;  // row of D: shift row / (8 GC), output channel row % (8 GC)
+      const int j = row / (8 * GC), o = row % (8 * GC);
+      if ((row & ~31) >= 72 * GC) break;  // no warp past the ninth copy has anything to add
+#pragma unroll 1
+      for (int c = 0; c < S::kN; c += 16) {
+        uint32_t v[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+            : "r"(tmem + ((uint32_t)(32 * w) << 16) + m * S::kN + c)
+            : "memory");
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (j < 9) {
+          float* dst = out + ((size_t)((c / CI) * 9 + j) * CI + c % CI) * LO + o;
+#pragma unroll
+          for (int k = 0; k < 16; ++k) atomicAdd(dst + k * LO, __uint_as_float(v[k]));
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (w == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::kCols) : "memory");
+}
+
+// gb[o] += sum_s gy[s, o] for the first NO of gy's LG channels: 16-byte loads,
+// eight channels per thread (2-byte loads of one channel each: 34 us at 16^4,
+// now 4.5)
+template <int LG, int NO>
+__global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ gy, float* __restrict__ gb, int V) {
+  constexpr int Q = NO / 8, R = 256 / Q;  // threads per row, rows per pass
+  __shared__ float part[8][NO];
+  const int q = threadIdx.x % Q, r = threadIdx.x / Q;
+  float acc[8] = {};
+  for (int s = blockIdx.x * R + r; s < V; s += gridDim.x * R) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(gy + (size_t)s * LG + q * 8));
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      acc[2 * k] += __uint_as_float(u[k] << 16);
+      acc[2 * k + 1] += __uint_as_float(u[k] & 0xffff0000u);
+    }
+  }
+  // lanes of a warp with the same q, then the warps
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+#pragma unroll
+    for (int o = 16; o >= Q; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
+  if ((threadIdx.x & 31) < Q)
+#pragma unroll
+    for (int k = 0; k < 8; ++k) part[threadIdx.x >> 5][q * 8 + k] = acc[k];
+  __syncthreads();
+  if (threadIdx.x < NO) {
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += part[k][threadIdx.x];
+    atomicAdd(gb + threadIdx.x, s);
   }
 }
 
@@ -748,14 +909,6 @@ __global__ void k_pack_weights(const float* __restrict__ p, bf16* __restrict__ W
   }
 }
 
-// flat gradient (parameter layout) from the padded last-layer gradient
-__global__ void k_unpad_grad3(const float* __restrict__ gW3p, const float* __restrict__ gb3p, float* __restrict__ gW3,
-                              float* __restrict__ gb3) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < 81 * kHid * kOut) gW3[i] = gW3p[(i / kOut) * kOutPad + i % kOut];
-  if (i < kOut) gb3[i] = gb3p[i];
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -785,28 +938,41 @@ cudaError_t launch_signal(const void* D, int V, float coef, void* gc, cudaStream
   return cudaPeekAtLastError();
 }
 
-cudaError_t launch_conv_bwd_weight(int layer, const void* x, const void* gy, float* gW, const Geom& geo,
-                                   cudaStream_t s) {
-  const int chunks = (int)(geo.V / 16);
-  const int cpw = 8;  // 16-site chunks per warp
-  dim3 grid((unsigned)((chunks + 4 * cpw - 1) / (4 * cpw)), 81);
-  const bf16* xp = static_cast<const bf16*>(x);
-  const bf16* gyp = static_cast<const bf16*>(gy);
-  if (layer == 1)
-    k_conv_bwd_weight<kFeat, kHid><<<grid, 128, 0, s>>>(xp, gyp, gW, geo, cpw);
-  else if (layer == 2)
-    k_conv_bwd_weight<kHid, kHid><<<grid, 128, 0, s>>>(xp, gyp, gW, geo, cpw);
-  else
-    k_conv_bwd_weight<kHid, kOutPad><<<grid, 128, 0, s>>>(xp, gyp, gW, geo, cpw);
+namespace {
+template <int CI, int GC, int LG, int LO>
+cudaError_t wgrad_launch(const void* x, const void* gy, float* gW, const Geom& geo, int* err, cudaStream_t s) {
+  using S = WgShape<CI, GC>;
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      k_wgrad_tc<CI, GC, LG, LO>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
+  if (attr != cudaSuccess) return attr;
+  const int64_t rows = (int64_t)(geo.L[0] + 2) * (geo.L[1] + 2) * geo.L[2] * geo.L[3];
+  const int nchunks = (int)((rows + kWgRows - 1) / kWgRows);
+  // three dt groups fill the 152 SMs with 50 CTAs each (100 where two fit an
+  // SM); a CTA takes at least four stages, so that its additions to gW
+  // (kMTiles x kN x 128, whatever its rows) stay a small part
+  const int most = S::kSmem <= 100 * 1024 ? 100 : 50;
+  int split = nchunks / 4;
+  split = split < 1 ? 1 : split > most ? most : split;
+  k_wgrad_tc<CI, GC, LG, LO><<<dim3((unsigned)split, 3), kTcThreads, S::kSmem, s>>>(
+      static_cast<const bf16*>(x), static_cast<const bf16*>(gy), gW, geo, nchunks, err);
   return cudaPeekAtLastError();
 }
+}  // namespace
 
-cudaError_t launch_bias_grad(int co, const void* gy, float* gb, int V, cudaStream_t s) {
+cudaError_t launch_conv_bwd_weight(int layer, const void* x, const void* gy, float* gW, const Geom& geo, int* err,
+                                   cudaStream_t s) {
+  if (layer == 1) return wgrad_launch<kFeat, kHid / 8, kHid, kHid>(x, gy, gW, geo, err, s);
+  if (layer == 2) return wgrad_launch<kHid, kHid / 8, kHid, kHid>(x, gy, gW, geo, err, s);
+  return wgrad_launch<kHid, kOut / 8, kOutPad, kOut>(x, gy, gW, geo, err, s);
+}
+
+cudaError_t launch_bias_grad(int layer, const void* gy, float* gb, int V, cudaStream_t s) {
   const bf16* g = static_cast<const bf16*>(gy);
-  if (co == kHid)
-    k_bias_grad<kHid><<<120, 256, 0, s>>>(g, gb, V);
+  const unsigned nb = (unsigned)(V / 256 < 1 ? 1 : V / 256 > 304 ? 304 : V / 256);
+  if (layer < 3)
+    k_bias_grad<kHid, kHid><<<nb, 256, 0, s>>>(g, gb, V);
   else
-    k_bias_grad<kOutPad><<<120, 256, 0, s>>>(g, gb, V);
+    k_bias_grad<kOutPad, kOut><<<nb, 256, 0, s>>>(g, gb, V);
   return cudaPeekAtLastError();
 }
 
@@ -863,11 +1029,6 @@ cudaError_t launch_conv_bwd_data_tc(int layer, const void* gy, const void* W, co
                                     const Geom& geo, int* err, cudaStream_t s) {
   if (layer == 3) return conv_tc_launch<kOutPad, kHid, -1, false>(gy, W, nullptr, a, gx, nullptr, geo, false, err, s);
   return conv_tc_launch<kHid, kHid, -1, false>(gy, W, nullptr, a, gx, nullptr, geo, false, err, s);
-}
-
-cudaError_t launch_unpad_grad3(const float* gW3p, const float* gb3p, float* gW3, float* gb3, cudaStream_t s) {
-  k_unpad_grad3<<<nb128(81 * kHid * kOut), 128, 0, s>>>(gW3p, gb3p, gW3, gb3);
-  return cudaPeekAtLastError();
 }
 
 }  // namespace warm

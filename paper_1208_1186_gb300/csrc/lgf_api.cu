@@ -1129,8 +1129,6 @@ struct lgf_net_ctx {
   float* b1 = nullptr;
   float* b2 = nullptr;
   float* b3 = nullptr;
-  float* gW3p = nullptr;  // padded last-layer gradient
-  float* gb3p = nullptr;
   int64_t vmax = 0;
   void *x0 = nullptr, *a1 = nullptr, *a2 = nullptr, *y3 = nullptr, *gc = nullptr, *ga2 = nullptr, *ga1 = nullptr;
   float* c = nullptr;  // FP32 [V][16] outputs of the last layer
@@ -2134,10 +2132,7 @@ int lgf_net_create(unsigned long long seed, lgf_net* out) {
   n->b1 = static_cast<float*>(net_alloc(n, 32 * 4));
   n->b2 = static_cast<float*>(net_alloc(n, 32 * 4));
   n->b3 = static_cast<float*>(net_alloc(n, 16 * 4));
-  n->gW3p = static_cast<float*>(net_alloc(n, (size_t)81 * 32 * 16 * 4));
-  n->gb3p = static_cast<float*>(net_alloc(n, 16 * 4));
-  if (!n->p || !n->m || !n->v || !n->g || !n->W1 || !n->W2 || !n->W3 || !n->b1 || !n->b2 || !n->b3 || !n->gW3p ||
-      !n->gb3p || !n->Wt1 || !n->Wt2 || !n->Wt3 || !n->tc_err) {
+  if (!n->p || !n->m || !n->v || !n->g || !n->W1 || !n->W2 || !n->W3 || !n->b1 || !n->b2 || !n->b3 || !n->Wt1 || !n->Wt2 || !n->Wt3 || !n->tc_err) {
     std::string msg = "device allocation of the network failed";
     lgf_net_destroy(n);
     return nfail(nullptr, LGF_ERR_OOM, msg);
@@ -2226,21 +2221,18 @@ int lgf_net_train_step(lgf_net n, lgf_handle h, double lr, double* F_out, float*
   LGF_NCUDA(n, warm::launch_signal(h->e32.D, V, (float)(-1.0 / (24.0 * (double)V)), n->gc, s));
   const size_t P = warm::kParams;
   LGF_NCUDA(n, cudaMemsetAsync(n->g, 0, P * 4, s));
-  LGF_NCUDA(n, cudaMemsetAsync(n->gW3p, 0, (size_t)81 * 32 * 16 * 4, s));
-  LGF_NCUDA(n, cudaMemsetAsync(n->gb3p, 0, 16 * 4, s));
   // layer 3 (a2 -> c)
-  LGF_NCUDA(n, warm::launch_conv_bwd_weight(3, n->a2, n->gc, n->gW3p, h->geo, s));
-  LGF_NCUDA(n, warm::launch_bias_grad(16, n->gc, n->gb3p, V, s));
+  LGF_NCUDA(n, warm::launch_conv_bwd_weight(3, n->a2, n->gc, n->g + kOW3, h->geo, n->tc_err, s));
+  LGF_NCUDA(n, warm::launch_bias_grad(3, n->gc, n->g + kOB3, V, s));
   LGF_NCUDA(n, warm::launch_conv_bwd_data_tc(3, n->gc, n->W3, n->a2, n->ga2, h->geo, n->tc_err, s));
   // layer 2 (a1 -> a2)
-  LGF_NCUDA(n, warm::launch_conv_bwd_weight(2, n->a1, n->ga2, n->g + kOW2, h->geo, s));
-  LGF_NCUDA(n, warm::launch_bias_grad(32, n->ga2, n->g + kOB2, V, s));
+  LGF_NCUDA(n, warm::launch_conv_bwd_weight(2, n->a1, n->ga2, n->g + kOW2, h->geo, n->tc_err, s));
+  LGF_NCUDA(n, warm::launch_bias_grad(2, n->ga2, n->g + kOB2, V, s));
   LGF_NCUDA(n, warm::launch_conv_bwd_data_tc(2, n->ga2, n->W2, n->a1, n->ga1, h->geo, n->tc_err, s));
   // layer 1 (x0 -> a1)
-  LGF_NCUDA(n, warm::launch_conv_bwd_weight(1, n->x0, n->ga1, n->g, h->geo, s));
-  LGF_NCUDA(n, warm::launch_bias_grad(32, n->ga1, n->g + kOB1, V, s));
-  LGF_NCUDA(n, warm::launch_unpad_grad3(n->gW3p, n->gb3p, n->g + kOW3, n->g + kOB3, s));
-  h->launches += 14;
+  LGF_NCUDA(n, warm::launch_conv_bwd_weight(1, n->x0, n->ga1, n->g, h->geo, n->tc_err, s));
+  LGF_NCUDA(n, warm::launch_bias_grad(1, n->ga1, n->g + kOB1, V, s));
+  h->launches += 13;
   if (host_grad) LGF_NCUDA(n, cudaMemcpyAsync(host_grad, n->g, P * 4, cudaMemcpyDeviceToHost, s));
   if (lr > 0.0) {
     n->step += 1;

@@ -196,9 +196,10 @@ constexpr int kParams = 81 * 48 * 32 + 32 + 81 * 32 * 32 + 32 + 81 * 32 * 8 + 8;
 cudaError_t launch_features(int nc, const void* U0, void* x, const Geom& geo, cudaStream_t s);
 cudaError_t launch_expmap(int nc, const float* c, int ldc, void* G, int V, cudaStream_t s);
 cudaError_t launch_signal(const void* D, int V, float coef, void* gc, cudaStream_t s);
-cudaError_t launch_conv_bwd_weight(int layer, const void* x, const void* gy, float* gW, const Geom& geo,
+// weight gradient of a layer, added to gW [81][in][out] (err as for the convolutions); bias gradient
+cudaError_t launch_conv_bwd_weight(int layer, const void* x, const void* gy, float* gW, const Geom& geo, int* err,
                                    cudaStream_t s);
-cudaError_t launch_bias_grad(int co, const void* gy, float* gb, int V, cudaStream_t s);
+cudaError_t launch_bias_grad(int layer, const void* gy, float* gb, int V, cudaStream_t s);
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float c1,
                         float c2, float eps, cudaStream_t s);
 cudaError_t launch_pack_weights(const float* p, void* W1, void* W2, void* W3, float* b1, float* b2, float* b3,
@@ -211,7 +212,6 @@ cudaError_t launch_conv_fwd_tc(int layer, const void* x, const void* Wt, const f
                                const Geom& geo, int* err, cudaStream_t s);
 cudaError_t launch_conv_bwd_data_tc(int layer, const void* gy, const void* W, const void* a, void* gx,
                                     const Geom& geo, int* err, cudaStream_t s);
-cudaError_t launch_unpad_grad3(const float* gW3p, const float* gb3p, float* gW3, float* gb3, cudaStream_t s);
 }  // namespace warm
 
 // text returned by lgf_last_error(NULL) on this host thread
