@@ -18,7 +18,10 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblgf.so")
-SOURCES = ["k_links.cu", "k_links_fx.cu", "k_gauge_rep.cu", "k_fft.cu", "k_fft_axis.cu", "k_fft_plane.cu", "k_fft_zt.cu", "k_warm.cu", "k_tail.cu", "lgf_api.cu", "lgf_noalloc.cu"]
+SOURCES = ["k_links.cu", "k_links_fx.cu", "k_gauge_rep.cu", "k_fft.cu", "k_fft_any.cu", "k_zt_pairs.cu", "k_fft_axis.cu", "k_fft_plane.cu", "k_fft_zt.cu", "k_warm.cu", "k_tail.cu", "lgf_api.cu", "lgf_noalloc.cu"]
+# sources compiled once per part, with -D<macro>=<part>
+PARTS = {"k_fft_any.cu": ("LGF_ANY_PART", range(8)),
+         "k_zt_pairs.cu": ("LGF_PAIR_Z", (4, 6, 8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 64))}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -52,10 +55,12 @@ def build(verbose: bool = False, extra_flags=()) -> str:
     objs = []
     for src in SOURCES:
         s = os.path.join(CSRC, src)
-        o = os.path.join(BUILD, src.replace(".cu", ".o"))
-        objs.append(o)
-        if not _newer(o, [s] + hdrs):
-            jobs.append([cc, *ARCH, *FLAGS, *extra_flags, "-c", s, "-o", o])
+        macro, parts = PARTS.get(src, (None, (0,)))
+        for part in parts:
+            o = os.path.join(BUILD, src.replace(".cu", f"_{part}.o" if macro else ".o"))
+            objs.append(o)
+            if not _newer(o, [s] + hdrs):
+                jobs.append([cc, *ARCH, *FLAGS, *extra_flags, *([f"-D{macro}={part}"] if macro else []), "-c", s, "-o", o])
 
     def run(cmd):
         if verbose:
@@ -67,7 +72,7 @@ def build(verbose: bool = False, extra_flags=()) -> str:
             print(r.stdout + r.stderr, flush=True)
 
     if jobs:
-        with cf.ThreadPoolExecutor(max_workers=len(jobs)) as ex:
+        with cf.ThreadPoolExecutor(max_workers=min(len(jobs), 2 * (os.cpu_count() or 8))) as ex:
             list(ex.map(run, jobs))
     if jobs or not _newer(LIB, objs):
         tmp = LIB + ".tmp"

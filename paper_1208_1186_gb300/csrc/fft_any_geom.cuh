@@ -1,0 +1,52 @@
+// Geometry and launchers of the any-extent FFT kernels (fft_any.cuh).
+#pragma once
+
+#include "lgf_kernels.cuh"
+
+namespace lgf {
+namespace anyfft {
+
+// quotient by a run-time divisor d: exact for n < 2^32 / d with rcp = ceil(2^32 / d)
+struct Div {
+  unsigned d, rcp;
+};
+inline Div make_div(int d) { return {(unsigned)d, 0xFFFFFFFFu / (unsigned)d + 1u}; }
+__device__ __forceinline__ int quot(int n, const Div& v) { return v.d == 1 ? n : (int)__umulhi((unsigned)n, v.rcp); }
+
+struct XyGeom {
+  int Lx, Ly, P, N;  // extents, padded row pitch, Lx Ly
+  int V, ntiles, tpc;  // sites, (plane, field) tiles, tiles per CTA
+  Div x;               // by Lx
+};
+
+struct ZtGeom {
+  int Lx, Ly, Lz, Lt;
+  int S, V;       // Lx Ly columns, sites
+  int bx, lbx;    // columns per tile (a power of two) and its logarithm
+  int PT;         // padded t pitch of a tile
+  Div x;          // by Lx
+};
+
+constexpr int kXyThreads = 128;
+
+// threads of a z-t CTA: bx max(Lz, Lt) at most
+template <class T, int kMaxLen>
+constexpr int zt_max_threads() {
+  return sizeof(T) == 4 && kMaxLen > 32 ? 4 * kMaxLen : 128;
+}
+
+// the kernels for extents up to kMaxLen = 32 or 64
+template <class T, int kMaxLen>
+struct Xy {
+  static cudaError_t init(int smem);
+  static cudaError_t launch(void* D, const XyGeom& g, size_t smem, bool inverse, const DevState* st, cudaStream_t s);
+};
+template <class T, int kMaxLen>
+struct Zt {
+  static cudaError_t init(int smem);
+  static cudaError_t launch(void* D, const ZtGeom& g, size_t smem, int threads, const void* kfac, const float* s2p,
+                            float c_over_V, const DevState* st, cudaStream_t s);
+};
+
+}  // namespace anyfft
+}  // namespace lgf

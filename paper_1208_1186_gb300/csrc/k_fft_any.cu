@@ -1,0 +1,28 @@
+// Instances of the any-extent FFT kernels (fft_any.cuh).  This file is
+// compiled once per part (build.py), because one instance holds the line
+// transforms of up to 26 lengths.
+#include "fft_any.cuh"
+
+namespace lgf {
+namespace anyfft {
+
+#if LGF_ANY_PART == 0
+template struct Xy<float, 32>;
+#elif LGF_ANY_PART == 1
+template struct Xy<float, 64>;
+#elif LGF_ANY_PART == 2
+template struct Xy<double, 32>;
+#elif LGF_ANY_PART == 3
+template struct Xy<double, 64>;
+#elif LGF_ANY_PART == 4
+template struct Zt<float, 32>;
+#elif LGF_ANY_PART == 5
+template struct Zt<float, 64>;
+#elif LGF_ANY_PART == 6
+template struct Zt<double, 32>;
+#elif LGF_ANY_PART == 7
+template struct Zt<double, 64>;
+#endif
+
+}  // namespace anyfft
+}  // namespace lgf

@@ -2,13 +2,11 @@
 // 2D" split of the 4D transform (Sec. 2.2) and in-register line FFTs
 // (fft_reg.cuh):
 //
-//   k_plane_xy(fwd) -> k_plane_zt(fwd z, fwd t, x p2_max/(V p2), inv t, inv z)
-//   -> k_plane_xy(inv)
+//   x-y (fwd) -> k_plane_zt(fwd z, fwd t, x p2_max/(V p2), inv t, inv z)
+//   -> x-y (inv)
 //
-// k_plane_xy: one CTA per (z, t) plane; the four fields of the plane
-// (4 LX LY complex) are staged in shared memory by asynchronous copies (no
-// register staging, all loads in flight at once); one thread per x-line does
-// the x transforms, then one thread per y-line the y transforms.
+// k_plane_xy_warp, k_plane_xy_pair: the x-y transforms of a plane's field in
+// one warp or two.
 // k_plane_zt (k_fft_zt.cu): the (z, t) transforms with the acceleration
 // factor in between.
 //
@@ -26,86 +24,10 @@ namespace lgf {
 
 namespace {
 
-// x-y planes with L <= 32 take the warp-tile kernel
-constexpr bool kXyWarpTiles = true;
 // FP32 gauge representation: the inverse x-y pass is fused with the G update,
 // which loads G for kXyGstepSites sites at a time
 constexpr bool kFuseXyinvGstep = true;
 constexpr int kXyGstepSites = 4;
-
-template <int LX, int LY>
-constexpr int xy_threads() {
-  return 4 * (LX > LY ? LX : LY);
-}
-
-// resident CTAs per SM asked of the register allocator: 4 x 128 threads at
-// up to 128 registers for lines up to 32 complex in FP32
-template <class T, int LX>
-constexpr int xy_min_blocks() {
-  return (sizeof(T) == 4 && LX <= 32) ? 4 : 1;
-}
-
-template <class T, int LX, int LY>
-constexpr size_t xy_smem_bytes() {
-  return (size_t)4 * LY * (LX + 1) * sizeof(cx<T>);
-}
-
-template <class T, int LX, int LY, bool INV>
-__global__ void __launch_bounds__(xy_threads<LX, LY>(), xy_min_blocks<T, LX>()) k_plane_xy(cx<T>* __restrict__ D, int V,
-                                                                   const DevState* __restrict__ st) {
-  pdl_wait();
-  if (st != nullptr && st->done) return;
-  constexpr int NT = xy_threads<LX, LY>();
-  constexpr int P = LX + 1;
-  constexpr int N = LX * LY;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<T>* tile = reinterpret_cast<cx<T>*>(smem_raw);  // [f][y][x], row pitch P
-  const int plane = blockIdx.x * N;
-  // stage the 4 planes (each contiguous in its field)
-  static_assert((4 * N) % NT == 0, "tile must split evenly over the threads");
-  constexpr int PER = 4 * N / NT;
-#pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    const int i = threadIdx.x + NT * k;
-    const int f = i / N, q = i % N;
-    cp_async_elem(tile + ((f * LY + q / LX) * P + q % LX), D + (f * V + plane + q));
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  if (threadIdx.x < 4 * LY) {  // x lines
-    cx<T>* row = tile + threadIdx.x * P;
-    cx<T> v[LX];
-#pragma unroll
-    for (int p = 0; p < LX; ++p) v[p] = row[p];
-    if (INV)
-      regfft::inverse<T, LX>(v);
-    else
-      regfft::forward<T, LX>(v);
-#pragma unroll
-    for (int p = 0; p < LX; ++p) row[p] = v[p];
-  }
-  __syncthreads();
-  if (threadIdx.x < 4 * LX) {  // y lines
-    const int f = threadIdx.x / LX, x = threadIdx.x % LX;
-    cx<T>* col = tile + f * LY * P + x;
-    cx<T> v[LY];
-#pragma unroll
-    for (int p = 0; p < LY; ++p) v[p] = col[p * P];
-    if (INV)
-      regfft::inverse<T, LY>(v);
-    else
-      regfft::forward<T, LY>(v);
-#pragma unroll
-    for (int p = 0; p < LY; ++p) col[p * P] = v[p];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    const int i = threadIdx.x + NT * k;
-    const int f = i / N, q = i % N;
-    D[f * V + plane + q] = tile[(f * LY + q / LX) * P + q % LX];
-  }
-}
 
 // x-y planes with L <= 32: a group of L lanes owns one (plane, field)
 // tile from its load to its store, so a warp needs no CTA barrier and warps
@@ -118,7 +40,7 @@ __global__ void __launch_bounds__(xy_threads<LX, LY>(), xy_min_blocks<T, LX>()) 
 // per warp (L <= 32; lanes past the last whole group idle through the
 // transforms).
 template <class T, int L>
-constexpr int xyw_smem_bytes() {
+constexpr int xyw_smem_bytes() {  // at most 17 KB, below the 48 KB that need no attribute
   return (32 / L) * L * (L + 1) * (int)sizeof(cx<T>);
 }
 
@@ -403,31 +325,29 @@ constexpr size_t xyinv_gstep_pair_smem() {
 
 namespace {
 
-// instantiated x-y planes (LX = LY) and z-t planes (LZ, LT), per precision
-#define LGF_XY_F32(X) X(4) X(6) X(8) X(12) X(16) X(20) X(24) X(32) X(48)
+// instantiated x-y planes (LX = LY), per precision: those of pipeline 3 and
+// those that only pipeline 1 uses
+#define LGF_XY_F32_P3(X) X(4) X(6) X(8) X(12) X(16) X(20) X(24) X(32) X(48)
+#define LGF_XY_F32_P1(X) X(10) X(18) X(30) X(36) X(40)
+#define LGF_XY_F32(X) LGF_XY_F32_P3(X) LGF_XY_F32_P1(X)
 #define LGF_XY_F64(X) X(4) X(6) X(8) X(12) X(16) X(20) X(24) X(32)
+// FP32 planes by the tile of one warp or of two
+#define LGF_XY_WARP(X) X(4) X(6) X(8) X(10) X(12) X(16) X(18) X(20) X(24) X(30) X(32)
+#define LGF_XY_TWO(X) X(36) X(40) X(48)
 template <class T, int L>
 cudaError_t xy_launch(void* D, int64_t V, int inverse, const DevState* st, cudaStream_t s, int Lz, int Lt) {
-  if constexpr (L <= 32 && kXyWarpTiles) {
-    const int ntiles = 4 * Lz * Lt;
+  const int ntiles = 4 * Lz * Lt;
+  const auto Dp = static_cast<cx<T>*>(D);
+  if constexpr (L <= 32) {
     const unsigned nb = (unsigned)((ntiles + 32 / L - 1) / (32 / L));
     constexpr int sm = xyw_smem_bytes<T, L>();
-    const auto Dp = static_cast<cx<T>*>(D);
     if (inverse) return launch_pdl(k_plane_xy_warp<T, L, true>, nb, 32, sm, s, Dp, (int)V, ntiles, st);
     return launch_pdl(k_plane_xy_warp<T, L, false>, nb, 32, sm, s, Dp, (int)V, ntiles, st);
-  } else if constexpr (L > 32 && L <= 64 && kXyWarpTiles) {
-    const int ntiles = 4 * Lz * Lt;
+  } else {
     constexpr int sm = L * (L + 1) * (int)sizeof(cx<T>);
-    const auto Dp = static_cast<cx<T>*>(D);
     if (inverse) return launch_pdl(k_plane_xy_pair<T, L, true>, (unsigned)ntiles, 64, sm, s, Dp, (int)V, ntiles, st);
     return launch_pdl(k_plane_xy_pair<T, L, false>, (unsigned)ntiles, 64, sm, s, Dp, (int)V, ntiles, st);
   }
-  const unsigned nb = (unsigned)(Lz * Lt);
-  constexpr int NT = xy_threads<L, L>();
-  constexpr size_t sm = xy_smem_bytes<T, L, L>();
-  const auto Dp = static_cast<cx<T>*>(D);
-  if (inverse) return launch_pdl(k_plane_xy<T, L, L, true>, nb, NT, sm, s, Dp, (int)V, st);
-  return launch_pdl(k_plane_xy<T, L, L, false>, nb, NT, sm, s, Dp, (int)V, st);
 }
 
 template <int L>
@@ -473,24 +393,6 @@ cudaError_t xyinv_gstep_launch(int nc, bool r64, const cx<float>* D, cx<float>* 
   return launch_pdl(k_plane_xyinv_gstep<L, 6, float, kXyGstepSites>, nb, 128, sm, s, D, G, V, nplanes, ha, st);
 }
 
-template <class T, int L>
-cudaError_t xy_attr() {
-  if constexpr (L <= 32) {
-    cudaError_t e = cudaFuncSetAttribute(k_plane_xy_warp<T, L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         xyw_smem_bytes<T, L>());
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_plane_xy_warp<T, L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               xyw_smem_bytes<T, L>());
-    if (e != cudaSuccess) return e;
-  }
-  cudaError_t e = cudaFuncSetAttribute(k_plane_xy<T, L, L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)xy_smem_bytes<T, L, L>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_plane_xy<T, L, L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)xy_smem_bytes<T, L, L>());
-  return e;
-}
-
 }  // namespace
 
 bool plane_pipeline_supported(int prec, int Lx, int Ly, int Lz, int Lt) {
@@ -500,7 +402,7 @@ bool plane_pipeline_supported(int prec, int Lx, int Ly, int Lz, int Lt) {
 #define LGF_XYQ(L) xy = xy || Lx == L;
 #define LGF_ZTQ(A, B) zt = zt || (Lz == A && Lt == B);
   if (prec == 4) {
-    LGF_XY_F32(LGF_XYQ)
+    LGF_XY_F32_P3(LGF_XYQ)
     LGF_ZT_F32(LGF_ZTQ)
   } else {
     LGF_XY_F64(LGF_XYQ)
@@ -513,15 +415,10 @@ bool plane_pipeline_supported(int prec, int Lx, int Ly, int Lz, int Lt) {
 
 cudaError_t plane_pipeline_init() {
   cudaError_t e = cudaSuccess;
-#define LGF_XYA32(L) \
-  if (e == cudaSuccess) e = xy_attr<float, L>();
-#define LGF_XYA64(L) \
-  if (e == cudaSuccess) e = xy_attr<double, L>();
-  if (e == cudaSuccess) e = xyinv_gstep_pair_attr<48>();
-  LGF_XY_F32(LGF_XYA32)
-  LGF_XY_F64(LGF_XYA64)
-#undef LGF_XYA32
-#undef LGF_XYA64
+#define LGF_TWO_ATTR(L) \
+  if (e == cudaSuccess) e = xyinv_gstep_pair_attr<L>();
+  LGF_XY_TWO(LGF_TWO_ATTR)
+#undef LGF_TWO_ATTR
   if (e == cudaSuccess) e = plane_zt_init();
   if (e == cudaSuccess) e = plane_xyinv_eta_init();
   return e;
@@ -543,14 +440,21 @@ cudaError_t launch_plane_xy(int prec, int L, void* D, int64_t V, int Lz, int Lt,
   return cudaErrorInvalidValue;
 }
 
-bool plane_xyinv_eta_supported(int L) {
-  switch (L) {
-    case 4: case 6: case 8: case 12: case 16: case 20: case 24: case 32:
-      return kFuseXyinvGstep;
-    default:
-      return false;
+bool plane_xy_supported(int prec, int Lx, int Ly) {
+  if (Lx != Ly) return false;
+  bool ok = false;
+#define LGF_XYQ(L) ok = ok || Lx == L;
+  if (prec == 4) {
+    LGF_XY_F32(LGF_XYQ)
+  } else {
+    LGF_XY_F64(LGF_XYQ)
+    ok = ok && 32 % Lx == 0;  // idle lanes waste the FP64 pipe
   }
+#undef LGF_XYQ
+  return ok;
 }
+
+bool plane_xyinv_eta_supported(int L) { return kFuseXyinvGstep && L <= 32 && plane_xy_supported(4, L, L); }
 
 cudaError_t plane_xyinv_eta_init() {
   cudaError_t e = cudaSuccess;
@@ -558,8 +462,7 @@ cudaError_t plane_xyinv_eta_init() {
   if (e == cudaSuccess)                                                                           \
     e = cudaFuncSetAttribute(k_plane_xyinv_eta<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                              (int)xyinv_gstep_smem<L>());
-  LGF_ETA_ATTR(4) LGF_ETA_ATTR(6) LGF_ETA_ATTR(8) LGF_ETA_ATTR(12) LGF_ETA_ATTR(16) LGF_ETA_ATTR(20) LGF_ETA_ATTR(24)
-  LGF_ETA_ATTR(32)
+  LGF_XY_WARP(LGF_ETA_ATTR)
 #undef LGF_ETA_ATTR
   return e;
 }
@@ -577,7 +480,7 @@ cudaError_t launch_plane_xyinv_eta(int L, const void* D, void* eta, int64_t V, i
                       h, st);                                                                                     \
   }
   switch (L) {
-    LGF_ETA_L(4) LGF_ETA_L(6) LGF_ETA_L(8) LGF_ETA_L(12) LGF_ETA_L(16) LGF_ETA_L(20) LGF_ETA_L(24) LGF_ETA_L(32)
+    LGF_XY_WARP(LGF_ETA_L)
     default:
       return cudaErrorInvalidValue;
   }
@@ -585,13 +488,7 @@ cudaError_t launch_plane_xyinv_eta(int L, const void* D, void* eta, int64_t V, i
 }
 
 bool plane_xyinv_gstep_supported(int prec, int L) {
-  if (!kFuseXyinvGstep || prec != 4) return false;
-  switch (L) {
-    case 4: case 6: case 8: case 12: case 16: case 20: case 24: case 32: case 48:
-      return true;
-    default:
-      return false;
-  }
+  return kFuseXyinvGstep && prec == 4 && plane_xy_supported(4, L, L);
 }
 
 cudaError_t launch_plane_xyinv_gstep(int L, int nc, const void* D, void* G, int64_t V, int Lz, int Lt,
@@ -600,15 +497,14 @@ cudaError_t launch_plane_xyinv_gstep(int L, int nc, const void* D, void* G, int6
   const auto Dp = static_cast<const cx<float>*>(D);
   const auto Gp = static_cast<cx<float>*>(G);
   switch (L) {
-    case 4: return xyinv_gstep_launch<4>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
-    case 6: return xyinv_gstep_launch<6>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
-    case 8: return xyinv_gstep_launch<8>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
-    case 12: return xyinv_gstep_launch<12>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
-    case 16: return xyinv_gstep_launch<16>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
-    case 20: return xyinv_gstep_launch<20>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
-    case 24: return xyinv_gstep_launch<24>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
-    case 32: return xyinv_gstep_launch<32>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
-    case 48: return xyinv_gstep_pair_launch<48>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
+#define LGF_GSTEP_L(N) \
+  case N: return xyinv_gstep_launch<N>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
+#define LGF_GSTEP_TWO(N) \
+  case N: return xyinv_gstep_pair_launch<N>(nc, reunit_fp64, Dp, Gp, (int)V, nplanes, half_alpha, st, s);
+    LGF_XY_WARP(LGF_GSTEP_L)
+    LGF_XY_TWO(LGF_GSTEP_TWO)
+#undef LGF_GSTEP_L
+#undef LGF_GSTEP_TWO
     default: return cudaErrorInvalidValue;
   }
 }

@@ -23,126 +23,11 @@
 // digit-reversed positions: s2p holds, per radix order, 4 sin^2 of the
 // frequency at each position of each axis (x and y always from order 0, the
 // x-y pass's order; for order 2, the z factor at each z slot of the tile).
-#include "fft_reg.cuh"
-#include "lgf_kernels.cuh"
+#include "zt_plane.cuh"
 
 namespace lgf {
 
 namespace {
-
-// pitch of one t slice: BX*LZ plus padding that shifts consecutive t slices
-// by one run of BX elements across the 32 shared-memory banks
-template <class T, int LZ, int BX>
-constexpr int zt_pitch() {
-  constexpr int W = (int)sizeof(cx<T>) / 4;  // banks per element
-  for (int pad = 0; pad < 32; ++pad)
-    if ((((BX * LZ + pad) * W) % 32) == ((BX * W) % 32)) return BX * LZ + pad;
-  return BX * LZ;
-}
-
-template <int LZ, int LT, int BX>
-constexpr int zt_threads() {
-  return BX * (LZ > LT ? LZ : LT);
-}
-
-// a thread holds a whole t line through the forward transform, the factor and
-// the inverse: FP32 lines up to 32 run 3 CTAs of 128 threads per SM at BX = 4
-// (up to 170 registers, no spills; 4 CTAs at 128 registers spilled 56 bytes
-// per thread and took 22.6 instead of 21.7 us at 32^4, 5 and 6 CTAs took
-// 23.9 and 28.9 us), 2 of 256 at BX = 8
-template <class T, int LZ, int LT, int BX>
-constexpr int zt_min_blocks() {
-  return (sizeof(T) == 4 && LZ <= 32 && LT <= 32) ? (BX <= 4 ? 3 : 2) : 1;
-}
-
-template <class T, int LZ, int LT, int BX>
-constexpr size_t zt_smem_bytes() {
-  return (size_t)zt_pitch<T, LZ, BX>() * LT * sizeof(cx<T>);
-}
-
-// FP32: factor from s2p[RO][axis][position] and c_over_V = p2_max / V, 0 at
-// k = 0.  FP64: per-site table kfac (an FP64 division per mode would be slow
-// on this GPU; FP64 runs radix order 0 only).
-template <class T, int LZ, int LT, int BX, int RO>
-__global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), zt_min_blocks<T, LZ, LT, BX>())
-    k_plane_zt(cx<T>* __restrict__ D, int Lx, int Ly, const T* __restrict__ kfac, const float* __restrict__ s2p,
-               float c_over_V, const DevState* __restrict__ st) {
-  pdl_wait();
-  if (st != nullptr && st->done) return;
-  constexpr int PT = zt_pitch<T, LZ, BX>();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<T>* tile = reinterpret_cast<cx<T>*>(smem_raw);  // [t][z][xb], t pitch PT
-  const int nxr = Lx / BX;
-  const int x0 = (blockIdx.x % nxr) * BX;
-  const int y = blockIdx.x / nxr;
-  const int f = blockIdx.y;
-  const int LxLy = Lx * Ly;
-  const int V = LxLy * LZ * LT;
-  cx<T>* Df = D + (f * V + x0 + Lx * y);
-  // forward z: line (xb, t) straight from global memory (for each z a warp
-  // reads BX consecutive x at 32 / BX values of t: whole 32-byte sectors)
-  if (threadIdx.x < BX * LT) {
-    const int xb = threadIdx.x % BX, t = threadIdx.x / BX;
-    cx<T>* line = tile + t * PT + xb;
-    const cx<T>* g = Df + (xb + LxLy * LZ * t);
-    cx<T> v[LZ];
-#pragma unroll
-    for (int p = 0; p < LZ; ++p) {  // running pointer: one address register
-      v[p] = *g;
-      g += LxLy;
-    }
-    regfft::forward<T, LZ, RO>(v);
-#pragma unroll
-    for (int p = 0; p < LZ; ++p) line[p * BX] = v[p];
-  }
-  __syncthreads();
-  // t lines (xb, z): forward, acceleration factor, inverse
-  if (threadIdx.x < BX * LZ) {
-    const int xb = threadIdx.x % BX, z = threadIdx.x / BX;
-    cx<T>* line = tile + z * BX + xb;
-    cx<T> v[LT];
-#pragma unroll
-    for (int p = 0; p < LT; ++p) v[p] = line[p * PT];
-    regfft::forward<T, LT, RO>(v);
-    const int x = x0 + xb;
-    if constexpr (sizeof(T) == 4) {
-      // the t contribution at each position is a compile-time constant
-      const float a = __ldg(s2p + x) + __ldg(s2p + kMaxL + y) + __ldg(s2p + RO * 4 * kMaxL + 2 * kMaxL + z);
-      const bool origin = (x | y | z) == 0;
-      regfft::static_for<0, LT>([&](auto pc) {
-        constexpr int p = decltype(pc)::value;
-        constexpr float s2t = (float)regfft::MomentumSq<LT, p, RO>::value;
-        float kf = c_over_V * rcp_approx(a + s2t);
-        if (p == 0 && origin) kf = 0.0f;
-        v[p] = scale(v[p], (T)kf);
-      });
-    } else {
-      static_assert(RO == 0, "FP64 z-t passes use radix order 0 (the per-site factor table's order)");
-      const T* kl = kfac + (x + Lx * (y + Ly * z));
-#pragma unroll
-      for (int p = 0; p < LT; ++p) v[p] = scale(v[p], __ldg(kl + p * (LxLy * LZ)));
-    }
-    regfft::inverse<T, LT, RO>(v);
-#pragma unroll
-    for (int p = 0; p < LT; ++p) line[p * PT] = v[p];
-  }
-  __syncthreads();
-  // inverse z, stored straight to global memory
-  if (threadIdx.x < BX * LT) {
-    const int xb = threadIdx.x % BX, t = threadIdx.x / BX;
-    const cx<T>* line = tile + t * PT + xb;
-    cx<T>* g = Df + (xb + LxLy * LZ * t);
-    cx<T> v[LZ];
-#pragma unroll
-    for (int p = 0; p < LZ; ++p) v[p] = line[p * BX];
-    regfft::inverse<T, LZ, RO>(v);
-#pragma unroll
-    for (int p = 0; p < LZ; ++p) {
-      *g = v[p];
-      g += LxLy;
-    }
-  }
-}
 
 // Radix order 2: the pair-split z and t transforms (FP32).  Thread 2 r + h
 // holds half h of line r.  The forward z transform leaves element p of half h
@@ -271,7 +156,7 @@ constexpr size_t zt_pair_smem_bytes() {
 template <class T, int LZ, int LT, int BX, int RO>
 cudaError_t zt_launch_one(void* D, int Lx, int Ly, const void* kfac, const float* s2p, float c_over_V,
                           const DevState* st, cudaStream_t s) {
-  dim3 grid((unsigned)((Lx / BX) * Ly), 4);
+  dim3 grid((unsigned)((Lx * Ly + BX - 1) / BX), 4);
   return launch_pdl(k_plane_zt<T, LZ, LT, BX, RO>, grid, zt_threads<LZ, LT, BX>(), zt_smem_bytes<T, LZ, LT, BX>(),
                     s, static_cast<cx<T>*>(D), Lx, Ly, static_cast<const T*>(kfac), s2p, c_over_V, st);
 }

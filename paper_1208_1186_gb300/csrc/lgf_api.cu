@@ -41,23 +41,21 @@ struct Allocator {
 };
 Allocator g_alloc;
 
-// Buffers of one working precision: links, packed gradient, gauge step,
-// twiddle factors.
+// Buffers of one working precision: links, packed gradient, gauge step.
 struct Engine {
   int prec = 8;  // bytes per real: 8 (FP64) or 4 (FP32)
   int nc = 9;    // complex entries stored per matrix
   void* U = nullptr;
   void* D = nullptr;
   void* g = nullptr;
-  void* tw = nullptr;
-  FftGeom fg{};  // FFT tiling for this precision (plane pipeline)
   bool axis = false;     // per-axis register FFT passes apply to this lattice
   bool plane = false;    // three-pass register plane pipeline applies
   int tuned = 0;         // pipeline chosen by lgf_autotune or the tuning cache (0: none)
   int zt_bx = 0;         // plane pipeline: x-run width of the z-t tiles (0: default)
   int zt_ro = 0;         // plane pipeline: radix order of the z and t transforms
   bool grep = false;     // FP32 engine: gauge representation (U holds the loaded links, G is updated)
-  void* kfac = nullptr;  // axis pipeline, FP64: p2_max/(V p2(k)) per site, digit-reversed order
+  void* kfac = nullptr;  // FP64: p2_max/(V p2(k)) per site, digit-reversed order
+  double* s2d = nullptr;  // FP64: [4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions
   float* s2p = nullptr;  // FP32: [3][4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions of radix order 0, 1
                          // and at the tile slots of order 2 (the pair split)
   float c_over_V = 0.f;  // p2_max / V
@@ -95,7 +93,7 @@ struct lgf_ctx {
   double tail_theta = 1e-12;
   long long tail_max32 = -1;
   bool reunit_fp64 = false;   // FP32 storage: reunitarise g in FP64 arithmetic
-  int fft_pipeline = 0;       // 0 auto, 1 Stockham planes, 2 axis passes, 3 register planes
+  int fft_pipeline = 0;       // 0 auto, 1 any-extent planes, 2 axis passes, 3 register planes
   bool explicit_fp32 = false; // FP32 engine: update the links in place instead of G (from the next load)
   int exp_order = 1;          // g from 1 + alpha/2 Delta~ (1) or from its exact exponential (0)
   bool track_g = false;       // FP64 handles, from the next load: accumulate G <- g G (LGF_TRACK_G)
@@ -116,7 +114,6 @@ struct lgf_ctx {
   Engine* cur = nullptr;     // engine that holds the current links
   void* G = nullptr;         // mixed: accumulated gauge transformation (e32 storage)
   double* Uorig = nullptr;   // mixed: FP64 SoA copy of the loaded links (9 planes)
-  double* sin2 = nullptr;    // [4][kMaxL] 4 sin^2(pi k / L)
   double2* partial = nullptr;
   int nblk = 0;
   DevState* st = nullptr;    // device
@@ -234,75 +231,51 @@ int alloc_engine(lgf_handle h, Engine& e) {
   e.U = dev_alloc(h, (size_t)4 * e.nc * V * e.cbytes());
   e.D = dev_alloc(h, (size_t)4 * V * e.cbytes());
   e.g = dev_alloc(h, (size_t)9 * V * e.cbytes());
-  e.tw = dev_alloc(h, (size_t)4 * kMaxL * e.cbytes());
-  if (!e.U || !e.D || !e.g || !e.tw) return fail(h, LGF_ERR_OOM, "device allocation failed");
-  // twiddle factors e^{-2 pi i m / L} per axis, computed in long double
-  std::vector<double> tw64(8 * kMaxL, 0.0);
-  std::vector<float> tw32(8 * kMaxL, 0.0f);
-  for (int a = 0; a < 4; ++a) {
-    const int L = h->L[a];
-    for (int m = 0; m < L; ++m) {
-      const long double ang = 2.0L * 3.14159265358979323846264338327950288L * (long double)m / (long double)L;
-      const double c = (double)cosl(ang), s = (double)-sinl(ang);
-      tw64[2 * (a * kMaxL + m)] = c;
-      tw64[2 * (a * kMaxL + m) + 1] = s;
-      tw32[2 * (a * kMaxL + m)] = (float)c;
-      tw32[2 * (a * kMaxL + m) + 1] = (float)s;
-    }
-  }
-  if (e.prec == 8)
-    LGF_CUDA(h, cudaMemcpy(e.tw, tw64.data(), tw64.size() * sizeof(double), cudaMemcpyHostToDevice));
-  else
-    LGF_CUDA(h, cudaMemcpy(e.tw, tw32.data(), tw32.size() * sizeof(float), cudaMemcpyHostToDevice));
+  if (!e.U || !e.D || !e.g) return fail(h, LGF_ERR_OOM, "device allocation failed");
   e.axis = true;
   for (int a = 0; a < 4; ++a) e.axis = e.axis && axis_pass_supported(e.prec, h->L[a]);
   e.plane = plane_pipeline_supported(e.prec, h->L[0], h->L[1], h->L[2], h->L[3]);
-  if (e.axis || e.plane) {
-    // acceleration factor at every position the forward passes leave a mode:
-    // position p along an axis holds frequency digit_rev(L, p)
-    std::vector<double> s2[4];
-    std::vector<float> s2f(3 * 4 * kMaxL, 0.0f);
-    double p2max = 0.0;
-    for (int a = 0; a < 4; ++a) {
-      const int L = h->L[a];
-      s2[a].resize(L);
-      double m = 0.0;
-      for (int p = 0; p < L; ++p) {
-        const long double sk =
-            sinl(3.14159265358979323846264338327950288L * (long double)regfft::digit_rev(L, p) / (long double)L);
-        s2[a][p] = (double)(4.0L * sk * sk);
-        s2f[a * kMaxL + p] = (float)s2[a][p];
-        m = s2[a][p] > m ? s2[a][p] : m;
-        // the same at the positions of radix order 1
-        const long double sk1 = sinl(3.14159265358979323846264338327950288L *
-                                     (long double)regfft::digit_rev(L, p, 1) / (long double)L);
-        s2f[4 * kMaxL + a * kMaxL + p] = (float)(4.0L * sk1 * sk1);
-        // the pair split: slot 2 q + half holds frequency pair_freq(L, q, half)
-        if (regfft::pair_supported(L)) {
-          const long double sk2 = sinl(3.14159265358979323846264338327950288L *
-                                       (long double)regfft::pair_freq(L, p >> 1, p & 1) / (long double)L);
-          s2f[2 * 4 * kMaxL + a * kMaxL + p] = (float)(4.0L * sk2 * sk2);
-        }
+  // acceleration factor at every position the forward passes leave a mode:
+  // position p along an axis holds frequency digit_rev(L, p)
+  std::vector<double> s2[4];
+  std::vector<float> s2f(3 * 4 * kMaxL, 0.0f);
+  double p2max = 0.0;
+  for (int a = 0; a < 4; ++a) {
+    const int L = h->L[a];
+    s2[a].resize(L);
+    double m = 0.0;
+    for (int p = 0; p < L; ++p) {
+      const long double sk =
+          sinl(3.14159265358979323846264338327950288L * (long double)regfft::digit_rev(L, p) / (long double)L);
+      s2[a][p] = (double)(4.0L * sk * sk);
+      s2f[a * kMaxL + p] = (float)s2[a][p];
+      m = s2[a][p] > m ? s2[a][p] : m;
+      // the same at the positions of radix order 1
+      const long double sk1 = sinl(3.14159265358979323846264338327950288L *
+                                   (long double)regfft::digit_rev(L, p, 1) / (long double)L);
+      s2f[4 * kMaxL + a * kMaxL + p] = (float)(4.0L * sk1 * sk1);
+      // the pair split: slot 2 q + half holds frequency pair_freq(L, q, half)
+      if (regfft::pair_supported(L)) {
+        const long double sk2 = sinl(3.14159265358979323846264338327950288L *
+                                     (long double)regfft::pair_freq(L, p >> 1, p & 1) / (long double)L);
+        s2f[2 * 4 * kMaxL + a * kMaxL + p] = (float)(4.0L * sk2 * sk2);
       }
-      p2max += m;
     }
-    e.c_over_V = (float)(p2max / (double)V);
-    if (e.prec == 4) {
-      e.s2p = static_cast<float*>(dev_alloc(h, s2f.size() * sizeof(float)));
-      if (!e.s2p) return fail(h, LGF_ERR_OOM, "device allocation failed");
-      LGF_CUDA(h, cudaMemcpy(e.s2p, s2f.data(), s2f.size() * sizeof(float), cudaMemcpyHostToDevice));
-    } else {
-      e.kfac = dev_alloc(h, (size_t)V * e.prec);
-      if (!e.kfac) return fail(h, LGF_ERR_OOM, "device allocation failed");
-      std::vector<double> k64(V);
-      int64_t s = 0;
-      for (int t = 0; t < h->L[3]; ++t)
-        for (int z = 0; z < h->L[2]; ++z)
-          for (int y = 0; y < h->L[1]; ++y)
-            for (int x = 0; x < h->L[0]; ++x, ++s)
-              k64[s] = (x | y | z | t) ? p2max / ((s2[0][x] + s2[1][y] + s2[2][z] + s2[3][t]) * (double)V) : 0.0;
-      LGF_CUDA(h, cudaMemcpy(e.kfac, k64.data(), (size_t)V * 8, cudaMemcpyHostToDevice));
-    }
+    p2max += m;
+  }
+  e.c_over_V = (float)(p2max / (double)V);
+  if (e.prec == 4) {
+    e.s2p = static_cast<float*>(dev_alloc(h, s2f.size() * sizeof(float)));
+    if (!e.s2p) return fail(h, LGF_ERR_OOM, "device allocation failed");
+    LGF_CUDA(h, cudaMemcpy(e.s2p, s2f.data(), s2f.size() * sizeof(float), cudaMemcpyHostToDevice));
+  } else {
+    e.kfac = dev_alloc(h, (size_t)V * e.prec);
+    e.s2d = static_cast<double*>(dev_alloc(h, (size_t)4 * kMaxL * sizeof(double)));
+    if (!e.kfac || !e.s2d) return fail(h, LGF_ERR_OOM, "device allocation failed");
+    std::vector<double> t(4 * kMaxL, 0.0);
+    for (int a = 0; a < 4; ++a) std::copy(s2[a].begin(), s2[a].end(), t.begin() + a * kMaxL);
+    LGF_CUDA(h, cudaMemcpy(e.s2d, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
+    LGF_CUDA(h, launch_kfac(h->L, e.s2d, p2max, static_cast<double*>(e.kfac), h->stream));
   }
   return LGF_OK;
 }
@@ -362,47 +335,70 @@ int reset_state(lgf_handle h, double tol, int max_iter, bool with_hist, bool sta
   return LGF_OK;
 }
 
-// FFT pipeline for engine e: the register plane pipeline (3 passes) where
-// its shapes are instantiated, else the per-axis register passes (7), else
-// the shared-memory Stockham plane kernels; LGF_FFT_PIPELINE can force one
-// (falling back to Stockham where the forced one does not apply).
+// FFT pipeline for engine e, unless LGF_FFT_PIPELINE or a tuned schedule says
+// otherwise (a forced pipeline that does not apply falls back to 1):
+// 3, the plane kernels with tuned schedules, where the shape is instantiated;
+// else 1, plane passes of any extents, or 2, the per-axis register passes (7
+// launches), where they do better:
+//   FP32: only where a z or t extent has no z-t kernel of its own
+//   (32 x 16 x 16 x 64 before 64 had one: 111 against 134 us per update;
+//   16 x 24 x 32 x 32, which has: 88 against 81);
+//   FP64, bound by its pipe: pipeline 3 only where its tiles fill whole warps
+//   (20^4: 362 against 298 us), the per-axis passes, whose lines always do, from
+//   2^16 sites on (8 x 32^3: 425 against 445; 12 x 8 x 24 x 16: 97 against 96).
 int pick_pipeline(lgf_handle h, const Engine& e) {
   if (h->fft_pipeline == 0 && e.tuned != 0) return e.tuned;
   switch (h->fft_pipeline) {
     case 1: return 1;
     case 2: return e.axis ? 2 : 1;
     case 3: return e.plane ? 3 : 1;
-    default: return e.plane ? 3 : (e.axis ? 2 : 1);
+    default: break;
   }
+  if (e.plane && (e.prec == 4 || 32 % h->L[0] == 0)) return 3;
+  if (!e.axis || h->V < (1 << 16)) return 1;
+  return e.prec == 8 || !zt_pair_supported(4, h->L[2], h->L[3]) ? 2 : 1;
+}
+
+// The forward x-y and the z-t pass (with the acceleration factor) of the packed
+// gradient in e.D, by one of the plane pipelines.
+int queue_planes_forward(lgf_handle h, Engine& e, int pipe, const DevState* st) {
+  cudaStream_t s = h->stream;
+  const int* L = h->L;
+  if (pipe == 3) {
+    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(e.prec, L[0], e.D, h->V, L[2], L[3], 0, st, s));
+    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_plane_zt(e.prec, L[0], L[1], L[2], L[3], e.D, e.kfac, e.s2p, e.c_over_V,
+                                                e.zt_bx, e.zt_ro, st, s));
+  } else {
+    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_fft_xy(e.prec, L, e.D, 0, st, s));
+    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_fft_zt(e.prec, L, e.D, e.kfac, e.s2p, e.c_over_V, st, s));
+  }
+  return LGF_OK;
 }
 
 // Fourier acceleration of the packed gradient in e.D (forward 4D FFT, times
 // p2_max/(V p2), inverse).
 int queue_accelerate(lgf_handle h, Engine& e, const DevState* st) {
   cudaStream_t s = h->stream;
+  const int* L = h->L;
   const int pipe = pick_pipeline(h, e);
-  if (pipe == 3) {
-    const int* L = h->L;
-    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(e.prec, L[0], e.D, h->V, L[2], L[3], 0, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_plane_zt(e.prec, L[0], L[1], L[2], L[3], e.D, e.kfac, e.s2p, e.c_over_V,
-                                                e.zt_bx, e.zt_ro, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(e.prec, L[0], e.D, h->V, L[2], L[3], 1, st, s));
-  } else if (pipe == 2) {
-    const int64_t V = h->V;
-    const int64_t Sy = h->L[0], Sz = (int64_t)h->L[0] * h->L[1];
-    LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_xpass(e.prec, h->L[0], e.D, V, 0, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_strided(e.prec, h->L[1], e.D, V, Sy, 0, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_strided(e.prec, h->L[2], e.D, V, Sz, 0, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_T, launch_tpass(e.prec, h->L[3], e.D, V, h->L[0], h->L[1], e.kfac, e.s2p, e.c_over_V,
-                                            st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_strided(e.prec, h->L[2], e.D, V, Sz, 1, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_strided(e.prec, h->L[1], e.D, V, Sy, 1, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_xpass(e.prec, h->L[0], e.D, V, 1, st, s));
-  } else {
-    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_fft_xy(e.prec, e.D, e.fg, e.tw, 0, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_fft_zt(e.prec, e.D, e.fg, e.tw, h->sin2, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_fft_xy(e.prec, e.D, e.fg, e.tw, 1, st, s));
+  if (pipe != 2) {
+    int rc = queue_planes_forward(h, e, pipe, st);
+    if (rc) return rc;
+    if (pipe == 3)
+      LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(e.prec, L[0], e.D, h->V, L[2], L[3], 1, st, s));
+    else
+      LGF_LAUNCH(h, LGF_K_FFT_XY, launch_fft_xy(e.prec, L, e.D, 1, st, s));
+    return LGF_OK;
   }
+  const int64_t V = h->V;
+  const int64_t Sy = L[0], Sz = (int64_t)L[0] * L[1];
+  LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_xpass(e.prec, L[0], e.D, V, 0, st, s));
+  LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_strided(e.prec, L[1], e.D, V, Sy, 0, st, s));
+  LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_strided(e.prec, L[2], e.D, V, Sz, 0, st, s));
+  LGF_LAUNCH(h, LGF_K_FFT_T, launch_tpass(e.prec, L[3], e.D, V, L[0], L[1], e.kfac, e.s2p, e.c_over_V, st, s));
+  LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_strided(e.prec, L[2], e.D, V, Sz, 1, st, s));
+  LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_strided(e.prec, L[1], e.D, V, Sy, 1, st, s));
+  LGF_LAUNCH(h, LGF_K_FFT_AXIS, launch_xpass(e.prec, L[0], e.D, V, 1, st, s));
   return LGF_OK;
 }
 
@@ -481,13 +477,12 @@ int queue_iteration(lgf_handle h, Engine& e) {
     Engine& f = h->e32;
     LGF_LAUNCH(h, LGF_K_GRADIENT,
                launch_gradient_tail_eta(h->Udf, h->eta, h->tbase, f.D, h->partial, h->geo, h->st, 1, s));
-    if (pick_pipeline(h, f) == 3 && plane_xyinv_eta_supported(h->L[0])) {
+    const int pipe = pick_pipeline(h, f);
+    if (pipe != 2 && h->L[0] == h->L[1] && plane_xyinv_eta_supported(h->L[0])) {
       // forward x-y, z-t, then the inverse x-y pass fused with the eta step
       const int* L = h->L;
-      LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(f.prec, L[0], f.D, h->V, L[2], L[3], 0, h->st, s));
-      LGF_LAUNCH(h, LGF_K_FFT_ZT,
-                 launch_plane_zt(f.prec, L[0], L[1], L[2], L[3], f.D, f.kfac, f.s2p, f.c_over_V, f.zt_bx, f.zt_ro,
-                                 h->st, s));
+      int rc = queue_planes_forward(h, f, pipe, h->st);
+      if (rc) return rc;
       LGF_LAUNCH(h, LGF_K_XY_GSTEP,
                  launch_plane_xyinv_eta(L[0], f.D, h->eta, h->V, L[2], L[3], 0.5 * h->alpha, h->st, s));
       return LGF_OK;
@@ -520,13 +515,12 @@ int queue_iteration(lgf_handle h, Engine& e) {
   }
   int rc = queue_gradient(h, e, 1);
   if (rc) return rc;
-  if (e.grep && !exact && pick_pipeline(h, e) == 3 && plane_xyinv_gstep_supported(e.prec, h->L[0])) {
+  const int pipe = pick_pipeline(h, e);
+  if (e.grep && !exact && pipe != 2 && h->L[0] == h->L[1] && plane_xyinv_gstep_supported(e.prec, h->L[0])) {
     // forward x-y, z-t, then the inverse x-y fused with G <- g G
     const int* L = h->L;
-    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(e.prec, L[0], e.D, h->V, L[2], L[3], 0, h->st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_ZT,
-               launch_plane_zt(e.prec, L[0], L[1], L[2], L[3], e.D, e.kfac, e.s2p, e.c_over_V, e.zt_bx, e.zt_ro,
-                               h->st, s));
+    rc = queue_planes_forward(h, e, pipe, h->st);
+    if (rc) return rc;
     LGF_LAUNCH(h, LGF_K_XY_GSTEP, launch_plane_xyinv_gstep(L[0], e.nc, e.D, h->G, h->V, L[2], L[3], 0.5 * h->alpha,
                                                            h->reunit_fp64, h->st, s));
     return LGF_OK;
@@ -1266,14 +1260,11 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
   *out = nullptr;
   const int Ls[4] = {Lx, Ly, Lz, Lt};
   if (dtype < LGF_F64 || dtype > LGF_F64_R12) return fail(nullptr, LGF_ERR_ARG, "unknown dtype");
-  FftGeom fg{};
-  for (int a = 0; a < 4; ++a) {
-    if (!make_axis_plan(Ls[a], &fg.ax[a]))
+  for (int a = 0; a < 4; ++a)
+    if (Ls[a] < 2 || Ls[a] > kMaxL || !regfft::supported(Ls[a]))
       return fail(nullptr, LGF_ERR_ARG,
                   "each lattice extent must be in [2, 64] and a product of 2, 3 and 5; got " +
                       std::to_string(Ls[a]));
-    fg.L[a] = Ls[a];
-  }
   lgf_ctx* h = new (std::nothrow) lgf_ctx();
   if (!h) return fail(nullptr, LGF_ERR_OOM, "host allocation failed");
   h->dtype = dtype;
@@ -1288,17 +1279,6 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
   h->V = V;
   h->geo.V = V;
   geom_init_rcp(h->geo);
-  fg.V = V;
-  double p2max = 0.0;
-  for (int a = 0; a < 4; ++a) {
-    double m = 0.0;
-    for (int k = 0; k < Ls[a]; ++k) {
-      const double sk = sin(M_PI * (double)k / (double)Ls[a]);
-      m = fmax(m, 4.0 * sk * sk);
-    }
-    p2max += m;
-  }
-  fg.p2max = p2max;
   auto bail = [&](int code) {
     std::string msg = h->err;
     dev_free_all(h);
@@ -1322,29 +1302,11 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
     h->e32.prec = 4;
     h->e32.nc = (dtype == LGF_F32_R12) ? 6 : 9;
   }
-  // FFT tiling: Bx consecutive x (>= 32 bytes of complex data when Lx allows)
-  auto pick = [&](Engine& e) -> bool {
-    FftGeom g = fg;
-    const int want = e.prec == 8 ? 2 : 4;
-    int bx = 1;
-    for (int b = want; b >= 1; b >>= 1)
-      if (Lx % b == 0) {
-        bx = b;
-        break;
-      }
-    g.Bx = bx;
-    g.Pxy = Lx + 1;
-    g.Pt = bx * (Lz + 1);
-    e.fg = g;
-    return fft_xy_smem(g, e.prec) <= (size_t)smem_optin && fft_zt_smem(g, e.prec) <= (size_t)smem_optin;
-  };
-  if (!pick(h->e64) || (h->mixed && !pick(h->e32))) {
+  if (!extents_supported(h->L, 8, smem_optin) || (h->mixed && !extents_supported(h->L, 4, smem_optin))) {
     h->err = "lattice planes too large for the shared-memory FFT";
     return bail(LGF_ERR_ARG);
   }
-  // the opt-in limit is process-wide per kernel: always raise it to the device maximum
-  cudaError_t e = fft_set_smem_limits(8, smem_optin, smem_optin);
-  if (e == cudaSuccess) e = fft_set_smem_limits(4, smem_optin, smem_optin);
+  cudaError_t e = fft_any_init(smem_optin);
   if (e == cudaSuccess) e = axis_pass_init();
   if (e == cudaSuccess) e = plane_pipeline_init();
   if (e != cudaSuccess) {
@@ -1373,10 +1335,9 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
   h->nblk = gradient_blocks(V);
   h->partial = static_cast<double2*>(dev_alloc(h, (size_t)partial_capacity(V) * sizeof(double2)));
   h->st = static_cast<DevState*>(dev_alloc(h, sizeof(DevState)));
-  h->sin2 = static_cast<double*>(dev_alloc(h, 4 * kMaxL * sizeof(double)));
   h->hist_cap = 1 << 16;
   h->hist = static_cast<double*>(dev_alloc(h, (size_t)h->hist_cap * sizeof(double)));
-  if (!h->partial || !h->st || !h->sin2 || !h->hist) {
+  if (!h->partial || !h->st || !h->hist) {
     h->err = "device allocation failed";
     return bail(LGF_ERR_OOM);
   }
@@ -1384,16 +1345,6 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
     h->st_host = nullptr;
     h->err = "pinned host allocation failed";
     return bail(LGF_ERR_OOM);
-  }
-  std::vector<double> s2(4 * kMaxL, 0.0);
-  for (int a = 0; a < 4; ++a)
-    for (int k = 0; k < Ls[a]; ++k) {
-      const long double sk = sinl(3.14159265358979323846264338327950288L * (long double)k / (long double)Ls[a]);
-      s2[a * kMaxL + k] = (double)(4.0L * sk * sk);
-    }
-  if (cudaMemcpy(h->sin2, s2.data(), s2.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
-    h->err = "copy of the momentum table failed";
-    return bail(LGF_ERR_CUDA);
   }
   if (reset_state(h, -1.0, 0, false) || cudaStreamSynchronize(h->stream) != cudaSuccess) {
     h->err = "state initialisation failed";

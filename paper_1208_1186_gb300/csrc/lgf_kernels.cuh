@@ -33,43 +33,13 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 
 namespace lgf {
 
-constexpr int kMaxL = 64;       // longest lattice extent the on-chip FFT takes
-constexpr int kMaxStages = 6;   // radix stages per axis (4^3 = 64)
-
-// Mixed-radix factorisation of one axis, radix 4 first, then 2, 3, 5.
-struct AxisPlan {
-  int L;
-  int nst;
-  int radix[kMaxStages];
-};
-
-// Everything the FFT kernels need to know about the lattice.
-struct FftGeom {
-  AxisPlan ax[4];
-  int L[4];
-  int64_t V;
-  double p2max;   // sum_mu max_k 4 sin^2(pi k / L_mu)
-  int Bx;         // consecutive x per z-t CTA
-  int Pxy;        // padded row pitch of an x-y plane in shared memory
-  int Pt;         // padded pitch of one t slice of a z-t tile
-};
-
-bool make_axis_plan(int L, AxisPlan* p);
-
-// byte sizes of the dynamic shared memory each FFT kernel needs
-size_t fft_xy_smem(const FftGeom& fg, int real_bytes);
-size_t fft_zt_smem(const FftGeom& fg, int real_bytes);
-cudaError_t fft_set_smem_limits(int real_bytes, size_t xy, size_t zt);
+constexpr int kMaxL = 64;  // longest lattice extent
 
 // prec: 8 = FP64, 4 = FP32; nc: complex entries stored per matrix (9 or 6)
 // gradient + FP64 F/theta reduction (its last block finishes it); mode 0: F
 // and theta only, mode 1: also the stop decision of an iteration queue
 cudaError_t launch_gradient(int prec, int nc, const void* U, void* D, double2* partial,
                             const Geom& geo, DevState* st, int mode, cudaStream_t s);
-cudaError_t launch_fft_xy(int prec, void* D, const FftGeom& fg, const void* tw, int inverse,
-                          const DevState* st, cudaStream_t s);
-cudaError_t launch_fft_zt(int prec, void* D, const FftGeom& fg, const void* tw,
-                          const double* sin2, const DevState* st, cudaStream_t s);
 // exact: g from the exact exponential of alpha/2 Delta~ instead of 1 + alpha/2 Delta~
 cudaError_t launch_build_g(int prec, int nc, const void* D, void* g, int64_t V, double half_alpha,
                            bool reunit_fp64, bool exact, const DevState* st, cudaStream_t s);
@@ -109,6 +79,25 @@ cudaError_t launch_set_identity(int prec, int nc, void* G, int64_t V, cudaStream
 // packed gradient fields [4][V] -> [V][4] complex128 (for probes)
 cudaError_t launch_unpack_fields(int prec, const void* D, double* out, int64_t V, cudaStream_t s);
 
+// plane passes of any extents (k_fft.cu, fft_any.cuh): pipeline 1.
+// extents_supported: the lattices the library takes (products of 2, 3 and 5,
+// planes within the shared memory of one CTA)
+bool extents_supported(const int L[4], int prec, size_t smem_limit);
+cudaError_t fft_any_init(int smem);
+cudaError_t launch_fft_xy(int prec, const int L[4], void* D, int inverse, const DevState* st, cudaStream_t s);
+cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, const float* s2p, float c_over_V,
+                          const DevState* st, cudaStream_t s);
+
+// FP32 z-t kernels per pair of common extents (k_zt_pairs.cu)
+#define LGF_PAIR_EXTENTS(X) \
+  X(4) X(6) X(8) X(10) X(12) X(16) X(18) X(20) X(24) X(30) X(32) X(36) X(40) X(48) X(64)
+template <int LZ>
+cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* s2p, float c_over_V, const DevState* st,
+                           cudaStream_t s);
+bool zt_pair_supported(int prec, int Lz, int Lt);
+// kfac[s] = p2max / (V sum_a s2[a][x_a]), 0 at the origin; s2: [4][kMaxL]
+cudaError_t launch_kfac(const int L[4], const double* s2, double p2max, double* kfac, cudaStream_t s);
+
 // per-axis register FFT passes (k_fft_axis.cu); lengths 4..32 (FP64) and up
 // to 64 (FP32) with radices 4, 2, 3, 5
 bool axis_pass_supported(int prec, int L);
@@ -132,6 +121,8 @@ cudaError_t launch_tpass(int prec, int L, void* D, int64_t V, int Lx, int Ly, co
 bool plane_pipeline_supported(int prec, int Lx, int Ly, int Lz, int Lt);
 cudaError_t plane_pipeline_init();
 cudaError_t plane_zt_init();
+// x-y planes of equal extents with a kernel of their own (in FP64 those whose tiles fill a warp)
+bool plane_xy_supported(int prec, int Lx, int Ly);
 cudaError_t launch_plane_xy(int prec, int L, void* D, int64_t V, int Lz, int Lt, int inverse, const DevState* st,
                             cudaStream_t s);
 // z-t pass schedule: bx = x-run width of a tile (0: the default, 4 FP32 / 2
@@ -140,11 +131,11 @@ cudaError_t launch_plane_xy(int prec, int L, void* D, int64_t V, int Lz, int Lt,
 bool plane_zt_schedule_supported(int prec, int Lx, int Lz, int Lt, int bx, int ro);
 cudaError_t launch_plane_zt(int prec, int Lx, int Ly, int Lz, int Lt, void* D, const void* kfac, const float* s2p,
                             float c_over_V, int bx, int ro, const DevState* st, cudaStream_t s);
-// inverse x-y pass fused with G <- g G (FP32 gauge representation; Lx = Ly
-// one of 4, 6, 8, 12, 16, 20, 24, 32)
+// inverse x-y pass fused with G <- g G (FP32 gauge representation; every
+// Lx = Ly with an FP32 x-y kernel)
 bool plane_xyinv_gstep_supported(int prec, int L);
 // the double-float tail's inverse x-y pass fused with its eta step (FP32
-// packed gradient, Lx = Ly one of 4, 6, 8, 12, 16, 20, 24, 32)
+// packed gradient, Lx = Ly <= 32 with an x-y kernel)
 bool plane_xyinv_eta_supported(int L);
 cudaError_t plane_xyinv_eta_init();
 cudaError_t launch_plane_xyinv_eta(int L, const void* D, void* eta, int64_t V, int Lz, int Lt, double half_alpha,
