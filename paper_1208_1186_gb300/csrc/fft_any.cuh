@@ -129,7 +129,7 @@ __device__ __noinline__ void z_line_out(const cx<T>* line, int bx, cx<T>* dst, i
 // lines of kMaxLen complex numbers: as many CTAs as their registers leave
 template <class T, int kMaxLen>
 constexpr int xy_min_blocks() {
-  return sizeof(T) == 4 ? (kMaxLen <= 32 ? 4 : 2) : (kMaxLen <= 32 ? 2 : 1);
+  return sizeof(T) == 8 ? 1 : kMaxLen <= 32 ? 4 : 2;
 }
 
 // tpc tiles (one field of one (z, t) plane each: tile = 4 plane + field) per
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kXyThreads, (xy_min_blocks<T, kMaxLen>()))
 
 template <class T, int kMaxLen>
 constexpr int zt_min_blocks() {
-  return sizeof(T) == 4 && kMaxLen <= 32 ? 3 : sizeof(T) == 8 && kMaxLen > 32 ? 2 : 1;
+  return kMaxLen <= 32 ? 3 : 1;
 }
 
 // One CTA per field and run of bx consecutive (x, y) columns, whatever Lx: the

@@ -1,4 +1,5 @@
-// Geometry and launchers of the any-extent FFT kernels (fft_any.cuh).
+// Geometry and launchers of the any-extent FFT kernels (fft_any.cuh, and
+// fft_fx.cuh for FP64 lines up to 32).
 #pragma once
 
 #include "lgf_kernels.cuh"
@@ -32,10 +33,10 @@ constexpr int kXyThreads = 128;
 // threads of a z-t CTA: bx max(Lz, Lt) at most
 template <class T, int kMaxLen>
 constexpr int zt_max_threads() {
-  return sizeof(T) == 4 && kMaxLen > 32 ? 4 * kMaxLen : 128;
+  return sizeof(T) == 4 ? 4 * kMaxLen : 2 * kMaxLen;
 }
 
-// the kernels for extents up to kMaxLen = 32 or 64
+// the kernels for extents up to kMaxLen = 32 (FP32) or 64
 template <class T, int kMaxLen>
 struct Xy {
   static cudaError_t init(int smem);
@@ -49,4 +50,16 @@ struct Zt {
 };
 
 }  // namespace anyfft
+
+namespace fxfft {
+
+// the FP64 passes of extents up to 32 in block floating point (fft_fx.cuh)
+constexpr int kFxThreads = 128;
+cudaError_t init(int smem);
+cudaError_t launch_xy(void* D, const anyfft::XyGeom& g, size_t smem, int threads, bool inverse, const DevState* st,
+                      cudaStream_t s);
+cudaError_t launch_zt(void* D, const anyfft::ZtGeom& g, size_t smem, int threads, const double* kfac,
+                      int kmax_exponent, const DevState* st, cudaStream_t s);
+
+}  // namespace fxfft
 }  // namespace lgf

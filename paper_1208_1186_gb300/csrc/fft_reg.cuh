@@ -141,6 +141,12 @@ struct Twiddle {  // W_L^M = exp(-2 pi i M / L)
   static constexpr double im = -turn_cs(m, L, 1);
 };
 
+// v (wr + i wi)
+template <class T>
+__device__ __forceinline__ cx<T> mul_const(cx<T> v, T wr, T wi) {
+  return mk<T>(fmaT(v.re, wr, -v.im * wi), fmaT(v.re, wi, v.im * wr));
+}
+
 // v * W_L^M (CONJ: v * conj(W_L^M))
 template <class T, int L, int M, bool CONJ>
 __device__ __forceinline__ cx<T> mul_tw(cx<T> v) {
@@ -154,7 +160,7 @@ __device__ __forceinline__ cx<T> mul_tw(cx<T> v) {
   } else {
     constexpr T wr = (T)W::re;
     constexpr T wi = CONJ ? (T)-W::im : (T)W::im;
-    return mk<T>(fmaT(v.re, wr, -v.im * wi), fmaT(v.re, wi, v.im * wr));
+    return mul_const(v, wr, wi);  // by argument-dependent lookup for a type with its own product
   }
 }
 

@@ -13,7 +13,7 @@ using anyfft::XyGeom;
 using anyfft::ZtGeom;
 
 constexpr int kSms = 152;
-constexpr size_t kXyTileBytes = 48 * 1024;  // four CTAs share an SM's 227 KB
+constexpr size_t kXyTileBytes = 56 * 1024;  // four CTAs share an SM's 227 KB (three with tiles of up to 75 KB in FP64)
 
 // As many (plane, field) tiles per CTA as give its 128 threads a line each, if
 // four CTAs still fit an SM and every SM still gets a CTA.
@@ -107,32 +107,32 @@ bool extents_supported(const int L[4], int prec, size_t smem_limit) {
 cudaError_t fft_any_init(int smem) {
   cudaError_t e = anyfft::Xy<float, 32>::init(smem);
   if (e == cudaSuccess) e = anyfft::Xy<float, 64>::init(smem);
-  if (e == cudaSuccess) e = anyfft::Xy<double, 32>::init(smem);
+  if (e == cudaSuccess) e = fxfft::init(smem);
   if (e == cudaSuccess) e = anyfft::Xy<double, 64>::init(smem);
   if (e == cudaSuccess) e = anyfft::Zt<float, 32>::init(smem);
   if (e == cudaSuccess) e = anyfft::Zt<float, 64>::init(smem);
-  if (e == cudaSuccess) e = anyfft::Zt<double, 32>::init(smem);
   if (e == cudaSuccess) e = anyfft::Zt<double, 64>::init(smem);
   return e;
 }
 
 cudaError_t launch_fft_xy(int prec, const int L[4], void* D, int inverse, const DevState* st, cudaStream_t s) {
-  if (plane_xy_supported(prec, L[0], L[1]))
-    return launch_plane_xy(prec, L[0], D, (int64_t)L[0] * L[1] * L[2] * L[3], L[2], L[3], inverse, st, s);
+  if (prec == 4 && plane_xy_supported(L[0], L[1]))
+    return launch_plane_xy(L[0], D, (int64_t)L[0] * L[1] * L[2] * L[3], L[2], L[3], inverse, st, s);
   size_t sm = 0;
   const XyGeom g = xy_geom(prec, L, &sm);
   const int m = g.Lx > g.Ly ? g.Lx : g.Ly;
   const bool inv = inverse != 0;
   if (prec == 8) {
-    if (m <= 32) return anyfft::Xy<double, 32>::launch(D, g, sm, inv, st, s);
+    const int thr = g.tpc * m >= fxfft::kFxThreads ? fxfft::kFxThreads : (g.tpc * m + 31) & ~31;
+    if (m <= 32) return fxfft::launch_xy(D, g, sm, thr, inv, st, s);
     return anyfft::Xy<double, 64>::launch(D, g, sm, inv, st, s);
   }
   if (m <= 32) return anyfft::Xy<float, 32>::launch(D, g, sm, inv, st, s);
   return anyfft::Xy<float, 64>::launch(D, g, sm, inv, st, s);
 }
 
-cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, const float* s2p, float c_over_V,
-                          const DevState* st, cudaStream_t s) {
+cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, int kmax_exponent, const float* s2p,
+                          float c_over_V, const DevState* st, cudaStream_t s) {
   if (zt_pair_supported(prec, L[2], L[3])) {
     switch (L[2]) {
 #define LGF_CASE(N) \
@@ -146,7 +146,8 @@ cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, c
   const ZtGeom g = zt_geom(prec, L, &sm, &thr);
   const int m = g.Lz > g.Lt ? g.Lz : g.Lt;
   if (prec == 8) {
-    if (m <= 32) return anyfft::Zt<double, 32>::launch(D, g, sm, thr, kfac, s2p, c_over_V, st, s);
+    if (m <= 32)
+      return fxfft::launch_zt(D, g, sm, thr, static_cast<const double*>(kfac), kmax_exponent, st, s);
     return anyfft::Zt<double, 64>::launch(D, g, sm, thr, kfac, s2p, c_over_V, st, s);
   }
   if (m <= 32) return anyfft::Zt<float, 32>::launch(D, g, sm, thr, kfac, s2p, c_over_V, st, s);

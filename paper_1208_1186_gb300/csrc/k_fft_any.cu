@@ -1,4 +1,4 @@
-// Instances of the any-extent FFT kernels (fft_any.cuh).  This file is
+// Instances of the run-time any-extent FFT kernels (fft_any.cuh).  This file is
 // compiled once per part (build.py), because one instance holds the line
 // transforms of up to 26 lengths.
 #include "fft_any.cuh"
@@ -8,19 +8,12 @@ namespace anyfft {
 
 #if LGF_ANY_PART == 0
 template struct Xy<float, 32>;
+template struct Zt<float, 32>;
 #elif LGF_ANY_PART == 1
 template struct Xy<float, 64>;
-#elif LGF_ANY_PART == 2
-template struct Xy<double, 32>;
-#elif LGF_ANY_PART == 3
-template struct Xy<double, 64>;
-#elif LGF_ANY_PART == 4
-template struct Zt<float, 32>;
-#elif LGF_ANY_PART == 5
 template struct Zt<float, 64>;
-#elif LGF_ANY_PART == 6
-template struct Zt<double, 32>;
-#elif LGF_ANY_PART == 7
+#elif LGF_ANY_PART == 2
+template struct Xy<double, 64>;
 template struct Zt<double, 64>;
 #endif
 

@@ -330,6 +330,7 @@ namespace {
 #define LGF_XY_F32_P3(X) X(4) X(6) X(8) X(12) X(16) X(20) X(24) X(32) X(48)
 #define LGF_XY_F32_P1(X) X(10) X(18) X(30) X(36) X(40)
 #define LGF_XY_F32(X) LGF_XY_F32_P3(X) LGF_XY_F32_P1(X)
+// FP64 planes that pipeline 3 takes (fft_fx.cuh runs them)
 #define LGF_XY_F64(X) X(4) X(6) X(8) X(12) X(16) X(20) X(24) X(32)
 // FP32 planes by the tile of one warp or of two
 #define LGF_XY_WARP(X) X(4) X(6) X(8) X(10) X(12) X(16) X(18) X(20) X(24) X(30) X(32)
@@ -424,37 +425,24 @@ cudaError_t plane_pipeline_init() {
   return e;
 }
 
-cudaError_t launch_plane_xy(int prec, int L, void* D, int64_t V, int Lz, int Lt, int inverse, const DevState* st,
+cudaError_t launch_plane_xy(int L, void* D, int64_t V, int Lz, int Lt, int inverse, const DevState* st,
                             cudaStream_t s) {
 #define LGF_XY32(N) \
   if (L == N) return xy_launch<float, N>(D, V, inverse, st, s, Lz, Lt);
-#define LGF_XY64(N) \
-  if (L == N) return xy_launch<double, N>(D, V, inverse, st, s, Lz, Lt);
-  if (prec == 4) {
-    LGF_XY_F32(LGF_XY32)
-  } else {
-    LGF_XY_F64(LGF_XY64)
-  }
+  LGF_XY_F32(LGF_XY32)
 #undef LGF_XY32
-#undef LGF_XY64
   return cudaErrorInvalidValue;
 }
 
-bool plane_xy_supported(int prec, int Lx, int Ly) {
-  if (Lx != Ly) return false;
+bool plane_xy_supported(int Lx, int Ly) {
   bool ok = false;
 #define LGF_XYQ(L) ok = ok || Lx == L;
-  if (prec == 4) {
-    LGF_XY_F32(LGF_XYQ)
-  } else {
-    LGF_XY_F64(LGF_XYQ)
-    ok = ok && 32 % Lx == 0;  // idle lanes waste the FP64 pipe
-  }
+  LGF_XY_F32(LGF_XYQ)
 #undef LGF_XYQ
-  return ok;
+  return ok && Lx == Ly;
 }
 
-bool plane_xyinv_eta_supported(int L) { return kFuseXyinvGstep && L <= 32 && plane_xy_supported(4, L, L); }
+bool plane_xyinv_eta_supported(int L) { return kFuseXyinvGstep && L <= 32 && plane_xy_supported(L, L); }
 
 cudaError_t plane_xyinv_eta_init() {
   cudaError_t e = cudaSuccess;
@@ -488,7 +476,7 @@ cudaError_t launch_plane_xyinv_eta(int L, const void* D, void* eta, int64_t V, i
 }
 
 bool plane_xyinv_gstep_supported(int prec, int L) {
-  return kFuseXyinvGstep && prec == 4 && plane_xy_supported(4, L, L);
+  return kFuseXyinvGstep && prec == 4 && plane_xy_supported(L, L);
 }
 
 cudaError_t launch_plane_xyinv_gstep(int L, int nc, const void* D, void* G, int64_t V, int Lz, int Lt,

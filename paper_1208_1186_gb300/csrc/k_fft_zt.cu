@@ -12,7 +12,7 @@
 // Two schedule choices are template parameters, searched per lattice shape
 // by the autotuner (lgf_autotune):
 //   BX  the x-run width of a tile: 4 or 8 FP32 complex numbers (32 or 64
-//       bytes per z load of a warp), 2 or 4 in FP64;
+//       bytes per z load of a warp);
 //   RO  the radix order of the z and t transforms (fft_reg.cuh): 0 greedy
 //       (32 = 4 4 2), 1 the same factors reversed (32 = 2 4 4), 2 the pair
 //       split (FP32): two threads share each line, the first radix-2 stage
@@ -124,27 +124,20 @@ __global__ void __launch_bounds__(zt_pair_threads<LZ, LT, BX>(), zt_pair_min_blo
   }
 }
 
-// the x-run widths instantiated per precision (the first is the default)
-template <class T>
-constexpr int zt_bx_default() {
-  return sizeof(T) == 4 ? 4 : 2;
-}
-template <class T>
-constexpr int zt_bx_wide() {
-  return 2 * zt_bx_default<T>();
-}
+// the x-run widths instantiated (the first is the default)
+constexpr int kB0 = 4, kB1 = 8;
 
 // radix order 1 is instantiated only where it changes the z or t stages
-template <class T, int LZ, int LT>
+template <int LZ, int LT>
 constexpr bool zt_has_ro1() {
-  return sizeof(T) == 4 && (regfft::orders_differ(LZ) || regfft::orders_differ(LT));
+  return regfft::orders_differ(LZ) || regfft::orders_differ(LT);
 }
 
-// radix order 2 (pair split) for FP32 lines with at least one extent >= 16
+// radix order 2 (pair split) for lines with at least one extent >= 16
 // (the shorter lines fit their registers anyway) and warp-aligned phases
-template <class T, int LZ, int LT>
+template <int LZ, int LT>
 constexpr bool zt_has_ro2() {
-  return sizeof(T) == 4 && (LZ >= 16 || LT >= 16) && regfft::pair_supported(LZ) && regfft::pair_supported(LT) &&
+  return (LZ >= 16 || LT >= 16) && regfft::pair_supported(LZ) && regfft::pair_supported(LT) &&
          (2 * 4 * LZ) % 32 == 0 && (2 * 4 * LT) % 32 == 0;
 }
 
@@ -153,12 +146,12 @@ constexpr size_t zt_pair_smem_bytes() {
   return (size_t)zt_pitch<float, LZ, BX>() * LT * sizeof(cx<float>);
 }
 
-template <class T, int LZ, int LT, int BX, int RO>
-cudaError_t zt_launch_one(void* D, int Lx, int Ly, const void* kfac, const float* s2p, float c_over_V,
-                          const DevState* st, cudaStream_t s) {
+template <int LZ, int LT, int BX, int RO>
+cudaError_t zt_launch_one(void* D, int Lx, int Ly, const float* s2p, float c_over_V, const DevState* st,
+                          cudaStream_t s) {
   dim3 grid((unsigned)((Lx * Ly + BX - 1) / BX), 4);
-  return launch_pdl(k_plane_zt<T, LZ, LT, BX, RO>, grid, zt_threads<LZ, LT, BX>(), zt_smem_bytes<T, LZ, LT, BX>(),
-                    s, static_cast<cx<T>*>(D), Lx, Ly, static_cast<const T*>(kfac), s2p, c_over_V, st);
+  return launch_pdl(k_plane_zt<LZ, LT, BX, RO>, grid, zt_threads<LZ, LT, BX>(), zt_smem_bytes<float, LZ, LT, BX>(), s,
+                    static_cast<cx<float>*>(D), Lx, Ly, s2p, c_over_V, st);
 }
 
 template <int LZ, int LT, int BX>
@@ -169,54 +162,52 @@ cudaError_t zt_launch_pair(void* D, int Lx, int Ly, const float* s2p, float c_ov
                     zt_pair_smem_bytes<LZ, LT, BX>(), s, static_cast<cx<float>*>(D), Lx, Ly, s2p, c_over_V, st);
 }
 
-template <class T, int LZ, int LT>
-cudaError_t zt_launch(void* D, int Lx, int Ly, const void* kfac, const float* s2p, float c_over_V, int bx, int ro,
-                      const DevState* st, cudaStream_t s) {
-  constexpr int B0 = zt_bx_default<T>(), B1 = zt_bx_wide<T>();
-  if (bx == 0) bx = B0;
-  if (bx != B0 && bx != B1) return cudaErrorInvalidValue;
+template <int LZ, int LT>
+cudaError_t zt_launch(void* D, int Lx, int Ly, const float* s2p, float c_over_V, int bx, int ro, const DevState* st,
+                      cudaStream_t s) {
+  if (bx == 0) bx = kB0;
+  if (bx != kB0 && bx != kB1) return cudaErrorInvalidValue;
   if (Lx % bx != 0) return cudaErrorInvalidValue;
   if (ro == 2) {
-    if constexpr (zt_has_ro2<T, LZ, LT>()) {
-      if (bx == B0) return zt_launch_pair<LZ, LT, B0>(D, Lx, Ly, s2p, c_over_V, st, s);
-      return zt_launch_pair<LZ, LT, B1>(D, Lx, Ly, s2p, c_over_V, st, s);
+    if constexpr (zt_has_ro2<LZ, LT>()) {
+      if (bx == kB0) return zt_launch_pair<LZ, LT, kB0>(D, Lx, Ly, s2p, c_over_V, st, s);
+      return zt_launch_pair<LZ, LT, kB1>(D, Lx, Ly, s2p, c_over_V, st, s);
     }
     return cudaErrorInvalidValue;
   }
   if (ro == 1) {
-    if constexpr (zt_has_ro1<T, LZ, LT>()) {
-      if (bx == B0) return zt_launch_one<T, LZ, LT, B0, 1>(D, Lx, Ly, kfac, s2p, c_over_V, st, s);
-      return zt_launch_one<T, LZ, LT, B1, 1>(D, Lx, Ly, kfac, s2p, c_over_V, st, s);
+    if constexpr (zt_has_ro1<LZ, LT>()) {
+      if (bx == kB0) return zt_launch_one<LZ, LT, kB0, 1>(D, Lx, Ly, s2p, c_over_V, st, s);
+      return zt_launch_one<LZ, LT, kB1, 1>(D, Lx, Ly, s2p, c_over_V, st, s);
     }
     return cudaErrorInvalidValue;
   }
   if (ro != 0) return cudaErrorInvalidValue;
-  if (bx == B0) return zt_launch_one<T, LZ, LT, B0, 0>(D, Lx, Ly, kfac, s2p, c_over_V, st, s);
-  return zt_launch_one<T, LZ, LT, B1, 0>(D, Lx, Ly, kfac, s2p, c_over_V, st, s);
+  if (bx == kB0) return zt_launch_one<LZ, LT, kB0, 0>(D, Lx, Ly, s2p, c_over_V, st, s);
+  return zt_launch_one<LZ, LT, kB1, 0>(D, Lx, Ly, s2p, c_over_V, st, s);
 }
 
-template <class T, int LZ, int LT, int BX, int RO>
+template <int LZ, int LT, int BX, int RO>
 cudaError_t zt_attr_one() {
-  return cudaFuncSetAttribute(k_plane_zt<T, LZ, LT, BX, RO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)zt_smem_bytes<T, LZ, LT, BX>());
+  return cudaFuncSetAttribute(k_plane_zt<LZ, LT, BX, RO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)zt_smem_bytes<float, LZ, LT, BX>());
 }
 
-template <class T, int LZ, int LT>
+template <int LZ, int LT>
 cudaError_t zt_attr() {
-  constexpr int B0 = zt_bx_default<T>(), B1 = zt_bx_wide<T>();
-  cudaError_t e = zt_attr_one<T, LZ, LT, B0, 0>();
-  if (e == cudaSuccess) e = zt_attr_one<T, LZ, LT, B1, 0>();
-  if constexpr (zt_has_ro1<T, LZ, LT>()) {
-    if (e == cudaSuccess) e = zt_attr_one<T, LZ, LT, B0, 1>();
-    if (e == cudaSuccess) e = zt_attr_one<T, LZ, LT, B1, 1>();
+  cudaError_t e = zt_attr_one<LZ, LT, kB0, 0>();
+  if (e == cudaSuccess) e = zt_attr_one<LZ, LT, kB1, 0>();
+  if constexpr (zt_has_ro1<LZ, LT>()) {
+    if (e == cudaSuccess) e = zt_attr_one<LZ, LT, kB0, 1>();
+    if (e == cudaSuccess) e = zt_attr_one<LZ, LT, kB1, 1>();
   }
-  if constexpr (zt_has_ro2<T, LZ, LT>()) {
+  if constexpr (zt_has_ro2<LZ, LT>()) {
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_plane_zt_pair<LZ, LT, B0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)zt_pair_smem_bytes<LZ, LT, B0>());
+      e = cudaFuncSetAttribute(k_plane_zt_pair<LZ, LT, kB0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)zt_pair_smem_bytes<LZ, LT, kB0>());
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_plane_zt_pair<LZ, LT, B1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)zt_pair_smem_bytes<LZ, LT, B1>());
+      e = cudaFuncSetAttribute(k_plane_zt_pair<LZ, LT, kB1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)zt_pair_smem_bytes<LZ, LT, kB1>());
   }
   return e;
 }
@@ -226,13 +217,9 @@ cudaError_t zt_attr() {
 cudaError_t plane_zt_init() {
   cudaError_t e = cudaSuccess;
 #define LGF_ZTA32(A, B) \
-  if (e == cudaSuccess) e = zt_attr<float, A, B>();
-#define LGF_ZTA64(A, B) \
-  if (e == cudaSuccess) e = zt_attr<double, A, B>();
+  if (e == cudaSuccess) e = zt_attr<A, B>();
   LGF_ZT_F32(LGF_ZTA32)
-  LGF_ZT_F64(LGF_ZTA64)
 #undef LGF_ZTA32
-#undef LGF_ZTA64
   return e;
 }
 
@@ -246,25 +233,18 @@ bool plane_zt_schedule_supported(int prec, int Lx, int Lz, int Lt, int bx, int r
   if (ro != 2) return false;
   bool inst = false;
 #define LGF_ZTR2(A, B) \
-  if (Lz == A && Lt == B) inst = zt_has_ro2<float, A, B>();
+  if (Lz == A && Lt == B) inst = zt_has_ro2<A, B>();
   LGF_ZT_F32(LGF_ZTR2)
 #undef LGF_ZTR2
   return inst;
 }
 
-cudaError_t launch_plane_zt(int prec, int Lx, int Ly, int Lz, int Lt, void* D, const void* kfac, const float* s2p,
-                            float c_over_V, int bx, int ro, const DevState* st, cudaStream_t s) {
+cudaError_t launch_plane_zt(int Lx, int Ly, int Lz, int Lt, void* D, const float* s2p, float c_over_V, int bx, int ro,
+                            const DevState* st, cudaStream_t s) {
 #define LGF_ZT32(A, B) \
-  if (Lz == A && Lt == B) return zt_launch<float, A, B>(D, Lx, Ly, kfac, s2p, c_over_V, bx, ro, st, s);
-#define LGF_ZT64(A, B) \
-  if (Lz == A && Lt == B) return zt_launch<double, A, B>(D, Lx, Ly, kfac, s2p, c_over_V, bx, ro, st, s);
-  if (prec == 4) {
-    LGF_ZT_F32(LGF_ZT32)
-  } else {
-    LGF_ZT_F64(LGF_ZT64)
-  }
+  if (Lz == A && Lt == B) return zt_launch<A, B>(D, Lx, Ly, s2p, c_over_V, bx, ro, st, s);
+  LGF_ZT_F32(LGF_ZT32)
 #undef LGF_ZT32
-#undef LGF_ZT64
   return cudaErrorInvalidValue;
 }
 

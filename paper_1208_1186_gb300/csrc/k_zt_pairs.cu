@@ -23,12 +23,12 @@ cudaError_t pair_launch(void* D, int Lx, int Ly, const float* s2p, float c_over_
   constexpr size_t sm = zt_smem_bytes<float, LZ, LT, BX>();
   if constexpr (sm > 48 * 1024) {  // once per process
     static const cudaError_t attr = cudaFuncSetAttribute(
-        k_plane_zt<float, LZ, LT, BX, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        k_plane_zt<LZ, LT, BX, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (attr != cudaSuccess) return attr;
   }
   dim3 grid((unsigned)((Lx * Ly + BX - 1) / BX), 4);
-  return launch_pdl(k_plane_zt<float, LZ, LT, BX, 0>, grid, zt_threads<LZ, LT, BX>(), sm, s,
-                    static_cast<cx<float>*>(D), Lx, Ly, static_cast<const float*>(nullptr), s2p, c_over_V, st);
+  return launch_pdl(k_plane_zt<LZ, LT, BX, 0>, grid, zt_threads<LZ, LT, BX>(), sm, s,
+                    static_cast<cx<float>*>(D), Lx, Ly, s2p, c_over_V, st);
 }
 
 }  // namespace

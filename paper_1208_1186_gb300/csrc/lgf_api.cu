@@ -55,6 +55,7 @@ struct Engine {
   int zt_ro = 0;         // plane pipeline: radix order of the z and t transforms
   bool grep = false;     // FP32 engine: gauge representation (U holds the loaded links, G is updated)
   void* kfac = nullptr;  // FP64: p2_max/(V p2(k)) per site, digit-reversed order
+  int kmax_exponent = 0;  // FP64: biased exponent of kfac's largest entry
   double* s2d = nullptr;  // FP64: [4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions
   float* s2p = nullptr;  // FP32: [3][4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions of radix order 0, 1
                          // and at the tile slots of order 2 (the pair split)
@@ -275,6 +276,12 @@ int alloc_engine(lgf_handle h, Engine& e) {
     std::vector<double> t(4 * kMaxL, 0.0);
     for (int a = 0; a < 4; ++a) std::copy(s2[a].begin(), s2[a].end(), t.begin() + a * kMaxL);
     LGF_CUDA(h, cudaMemcpy(e.s2d, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
+    // the largest factor is that of the smallest momentum
+    double p2min = p2max;
+    for (int a = 0; a < 4; ++a)
+      for (double s : s2[a])
+        if (s > 0.0 && s < p2min) p2min = s;
+    e.kmax_exponent = ilogb(p2max / (p2min * (double)V)) + 1023;
     LGF_CUDA(h, launch_kfac(h->L, e.s2d, p2max, static_cast<double*>(e.kfac), h->stream));
   }
   return LGF_OK;
@@ -337,15 +344,11 @@ int reset_state(lgf_handle h, double tol, int max_iter, bool with_hist, bool sta
 
 // FFT pipeline for engine e, unless LGF_FFT_PIPELINE or a tuned schedule says
 // otherwise (a forced pipeline that does not apply falls back to 1):
-// 3, the plane kernels with tuned schedules, where the shape is instantiated;
-// else 1, plane passes of any extents, or 2, the per-axis register passes (7
-// launches), where they do better:
-//   FP32: only where a z or t extent has no z-t kernel of its own
-//   (32 x 16 x 16 x 64 before 64 had one: 111 against 134 us per update;
-//   16 x 24 x 32 x 32, which has: 88 against 81);
-//   FP64, bound by its pipe: pipeline 3 only where its tiles fill whole warps
-//   (20^4: 362 against 298 us), the per-axis passes, whose lines always do, from
-//   2^16 sites on (8 x 32^3: 425 against 445; 12 x 8 x 24 x 16: 97 against 96).
+// 3, the FP32 plane kernels with tuned schedules, where the shape is
+// instantiated; else 1, plane passes of any extents.  The per-axis passes (2)
+// are seven launches, and every extent they take has plane kernels that beat
+// them (16 x 24 x 32 x 32: 88 against 81 us per update; 6 x 12 x 4 x 20: 27
+// against 21).  FP64 runs pipelines 1 and 3 by the same kernels.
 int pick_pipeline(lgf_handle h, const Engine& e) {
   if (h->fft_pipeline == 0 && e.tuned != 0) return e.tuned;
   switch (h->fft_pipeline) {
@@ -354,9 +357,7 @@ int pick_pipeline(lgf_handle h, const Engine& e) {
     case 3: return e.plane ? 3 : 1;
     default: break;
   }
-  if (e.plane && (e.prec == 4 || 32 % h->L[0] == 0)) return 3;
-  if (!e.axis || h->V < (1 << 16)) return 1;
-  return e.prec == 8 || !zt_pair_supported(4, h->L[2], h->L[3]) ? 2 : 1;
+  return e.plane ? 3 : 1;
 }
 
 // The forward x-y and the z-t pass (with the acceleration factor) of the packed
@@ -364,13 +365,13 @@ int pick_pipeline(lgf_handle h, const Engine& e) {
 int queue_planes_forward(lgf_handle h, Engine& e, int pipe, const DevState* st) {
   cudaStream_t s = h->stream;
   const int* L = h->L;
-  if (pipe == 3) {
-    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(e.prec, L[0], e.D, h->V, L[2], L[3], 0, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_plane_zt(e.prec, L[0], L[1], L[2], L[3], e.D, e.kfac, e.s2p, e.c_over_V,
-                                                e.zt_bx, e.zt_ro, st, s));
+  if (pipe == 3 && e.prec == 4) {
+    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(L[0], e.D, h->V, L[2], L[3], 0, st, s));
+    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_plane_zt(L[0], L[1], L[2], L[3], e.D, e.s2p, e.c_over_V, e.zt_bx, e.zt_ro, st,
+                                                s));
   } else {
     LGF_LAUNCH(h, LGF_K_FFT_XY, launch_fft_xy(e.prec, L, e.D, 0, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_fft_zt(e.prec, L, e.D, e.kfac, e.s2p, e.c_over_V, st, s));
+    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_fft_zt(e.prec, L, e.D, e.kfac, e.kmax_exponent, e.s2p, e.c_over_V, st, s));
   }
   return LGF_OK;
 }
@@ -384,10 +385,7 @@ int queue_accelerate(lgf_handle h, Engine& e, const DevState* st) {
   if (pipe != 2) {
     int rc = queue_planes_forward(h, e, pipe, st);
     if (rc) return rc;
-    if (pipe == 3)
-      LGF_LAUNCH(h, LGF_K_FFT_XY, launch_plane_xy(e.prec, L[0], e.D, h->V, L[2], L[3], 1, st, s));
-    else
-      LGF_LAUNCH(h, LGF_K_FFT_XY, launch_fft_xy(e.prec, L, e.D, 1, st, s));
+    LGF_LAUNCH(h, LGF_K_FFT_XY, launch_fft_xy(e.prec, L, e.D, 1, st, s));
     return LGF_OK;
   }
   const int64_t V = h->V;

@@ -85,8 +85,8 @@ cudaError_t launch_unpack_fields(int prec, const void* D, double* out, int64_t V
 bool extents_supported(const int L[4], int prec, size_t smem_limit);
 cudaError_t fft_any_init(int smem);
 cudaError_t launch_fft_xy(int prec, const int L[4], void* D, int inverse, const DevState* st, cudaStream_t s);
-cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, const float* s2p, float c_over_V,
-                          const DevState* st, cudaStream_t s);
+cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, int kmax_exponent, const float* s2p,
+                          float c_over_V, const DevState* st, cudaStream_t s);
 
 // FP32 z-t kernels per pair of common extents (k_zt_pairs.cu)
 #define LGF_PAIR_EXTENTS(X) \
@@ -105,7 +105,8 @@ cudaError_t axis_pass_init();
 cudaError_t launch_xpass(int prec, int L, void* D, int64_t V, int inverse, const DevState* st, cudaStream_t s);
 cudaError_t launch_strided(int prec, int L, void* D, int64_t V, int64_t S, int inverse, const DevState* st,
                            cudaStream_t s);
-// FP64: factor from the per-site table kfac; FP32: from s2p[axis][position]
+// FP64: factor from the per-site table kfac (kmax_exponent: the biased exponent of its largest entry); FP32:
+// from s2p[axis][position]
 // (4 sin^2 at the digit-reversed frequency) and c_over_V = p2_max / V
 cudaError_t launch_tpass(int prec, int L, void* D, int64_t V, int Lx, int Ly, const void* kfac, const float* s2p,
                          float c_over_V, const DevState* st, cudaStream_t s);
@@ -121,16 +122,17 @@ cudaError_t launch_tpass(int prec, int L, void* D, int64_t V, int Lx, int Ly, co
 bool plane_pipeline_supported(int prec, int Lx, int Ly, int Lz, int Lt);
 cudaError_t plane_pipeline_init();
 cudaError_t plane_zt_init();
-// x-y planes of equal extents with a kernel of their own (in FP64 those whose tiles fill a warp)
-bool plane_xy_supported(int prec, int Lx, int Ly);
-cudaError_t launch_plane_xy(int prec, int L, void* D, int64_t V, int Lz, int Lt, int inverse, const DevState* st,
+// FP32 x-y planes of equal extents with a kernel of their own
+bool plane_xy_supported(int Lx, int Ly);
+cudaError_t launch_plane_xy(int L, void* D, int64_t V, int Lz, int Lt, int inverse, const DevState* st,
                             cudaStream_t s);
-// z-t pass schedule: bx = x-run width of a tile (0: the default, 4 FP32 / 2
-// FP64; or twice that), ro = radix order of the z and t transforms (0, or 1
-// for FP32 where it changes the stages); s2p holds [2][4][kMaxL] FP32 factors
+// FP32 z-t pass schedule: bx = x-run width of a tile (0: the default, 4; or 8),
+// ro = radix order of the z and t transforms; s2p holds [3][4][kMaxL] factors.
+// FP64 takes bx = 0, 2 or 4 and ro = 0: its pass (fft_fx.cuh) has a tiling of
+// its own, and every schedule runs the same kernels.
 bool plane_zt_schedule_supported(int prec, int Lx, int Lz, int Lt, int bx, int ro);
-cudaError_t launch_plane_zt(int prec, int Lx, int Ly, int Lz, int Lt, void* D, const void* kfac, const float* s2p,
-                            float c_over_V, int bx, int ro, const DevState* st, cudaStream_t s);
+cudaError_t launch_plane_zt(int Lx, int Ly, int Lz, int Lt, void* D, const float* s2p, float c_over_V, int bx, int ro,
+                            const DevState* st, cudaStream_t s);
 // inverse x-y pass fused with G <- g G (FP32 gauge representation; every
 // Lx = Ly with an FP32 x-y kernel)
 bool plane_xyinv_gstep_supported(int prec, int L);

@@ -1,4 +1,4 @@
-// The z-t plane kernel of the plane pipelines (k_fft_zt.cu describes the pass
+// The FP32 z-t plane kernel of the plane pipelines (k_fft_zt.cu describes the pass
 // and instantiates the shapes with tuned schedules; k_zt_pairs.cu the other
 // pairs of common extents): one CTA per field and run of BX consecutive (x, y)
 // columns, which are contiguous at every (z, t) whatever Lx; a run may cross
@@ -30,9 +30,9 @@ constexpr int zt_threads() {
 // (up to 170 registers, no spills; 4 CTAs at 128 registers spilled 56 bytes
 // per thread and took 22.6 instead of 21.7 us at 32^4, 5 and 6 CTAs took
 // 23.9 and 28.9 us), 2 of 256 at BX = 8
-template <class T, int LZ, int LT, int BX>
+template <int LZ, int LT, int BX>
 constexpr int zt_min_blocks() {
-  return (sizeof(T) == 4 && LZ <= 32 && LT <= 32) ? (BX <= 4 ? 3 : 2) : 1;
+  return LZ <= 32 && LT <= 32 ? (BX <= 4 ? 3 : 2) : 1;
 }
 
 template <class T, int LZ, int LT, int BX>
@@ -41,12 +41,12 @@ constexpr size_t zt_smem_bytes() {
 }
 
 // FP32: factor from s2p[RO][axis][position] and c_over_V = p2_max / V, 0 at
-// k = 0.  FP64: per-site table kfac (an FP64 division per mode would be slow
-// on this GPU; FP64 runs radix order 0 only).
-template <class T, int LZ, int LT, int BX, int RO>
-__global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), zt_min_blocks<T, LZ, LT, BX>())
-    k_plane_zt(cx<T>* __restrict__ D, int Lx, int Ly, const T* __restrict__ kfac, const float* __restrict__ s2p,
-               float c_over_V, const DevState* __restrict__ st) {
+// k = 0
+template <int LZ, int LT, int BX, int RO>
+__global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), zt_min_blocks<LZ, LT, BX>())
+    k_plane_zt(cx<float>* __restrict__ D, int Lx, int Ly, const float* __restrict__ s2p, float c_over_V,
+               const DevState* __restrict__ st) {
+  using T = float;
   pdl_wait();
   if (st != nullptr && st->done) return;
   constexpr int PT = zt_pitch<T, LZ, BX>();
@@ -85,23 +85,16 @@ __global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), zt_min_blocks<T, LZ,
     for (int p = 0; p < LT; ++p) v[p] = line[p * PT];
     regfft::forward<T, LT, RO>(v);
     const int q = q0 + xb, y = q / Lx, x = q - y * Lx;
-    if constexpr (sizeof(T) == 4) {
-      // the t contribution at each position is a compile-time constant
-      const float a = __ldg(s2p + x) + __ldg(s2p + kMaxL + y) + __ldg(s2p + RO * 4 * kMaxL + 2 * kMaxL + z);
-      const bool origin = (x | y | z) == 0;
-      regfft::static_for<0, LT>([&](auto pc) {
-        constexpr int p = decltype(pc)::value;
-        constexpr float s2t = (float)regfft::MomentumSq<LT, p, RO>::value;
-        float kf = c_over_V * rcp_approx(a + s2t);
-        if (p == 0 && origin) kf = 0.0f;
-        v[p] = scale(v[p], (T)kf);
-      });
-    } else {
-      static_assert(RO == 0, "FP64 z-t passes use radix order 0 (the per-site factor table's order)");
-      const T* kl = kfac + (q + LxLy * z);
-#pragma unroll
-      for (int p = 0; p < LT; ++p) v[p] = scale(v[p], __ldg(kl + p * (LxLy * LZ)));
-    }
+    // the t contribution at each position is a compile-time constant
+    const float a = __ldg(s2p + x) + __ldg(s2p + kMaxL + y) + __ldg(s2p + RO * 4 * kMaxL + 2 * kMaxL + z);
+    const bool origin = (x | y | z) == 0;
+    regfft::static_for<0, LT>([&](auto pc) {
+      constexpr int p = decltype(pc)::value;
+      constexpr float s2t = (float)regfft::MomentumSq<LT, p, RO>::value;
+      float kf = c_over_V * rcp_approx(a + s2t);
+      if (p == 0 && origin) kf = 0.0f;
+      v[p] = scale(v[p], (T)kf);
+    });
     regfft::inverse<T, LT, RO>(v);
 #pragma unroll
     for (int p = 0; p < LT; ++p) line[p * PT] = v[p];
