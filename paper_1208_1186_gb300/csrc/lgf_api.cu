@@ -157,6 +157,13 @@ namespace {
 
 // lgf_fix without profiling runs each phase as one device-side graph loop
 constexpr bool kDeviceLoops = true;
+// Iterations per turn of a device-side loop: a turn of the while node costs about
+// 4 us (8^4: 23 us per update with one iteration per turn, 21 with two, 20 with
+// four).  More than two make the last turn's idle iterations and a new handle's
+// larger graph cost more than they save (8^4, first fix: four 922 us, one 903).
+// A batch keeps one, since its lanes overlap the turns and each call builds its
+// graph (sixteen of 16^4: 6.7 ms, with two 7.1).
+constexpr int kLoopUnroll = 2;
 
 int fail(lgf_handle h, int code, const std::string& msg) {
   if (h)
@@ -587,12 +594,12 @@ int build_loop(lgf_handle h, Engine& e, lgf_ctx::DevLoop& l) {
   int rc = LGF_OK;
   err = cudaStreamBeginCaptureToGraph(h->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (err == cudaSuccess) {
-    rc = queue_iteration(h, e);
+    for (int i = 0; i < kLoopUnroll && !rc; ++i) rc = queue_iteration(h, e);
     cudaGraph_t out = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &out);
     if (!rc && e2 != cudaSuccess) err = e2;
   }
-  l.launches = h->launches - l0;
+  l.launches = (h->launches - l0) / kLoopUnroll;
   h->launches = l0;
   h->stream = saved;
   if (!rc && err == cudaSuccess) err = cudaGraphInstantiate(&l.exec, g, 0);
