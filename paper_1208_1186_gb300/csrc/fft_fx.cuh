@@ -97,12 +97,13 @@ __device__ __forceinline__ int size_of_bits(long long bits, int E) {
   return sh < 32 ? (int)((((unsigned)hi & 0xfffffu) | 0x100000u) >> 3 >> sh) + 1 : 1;
 }
 
-// f 2^X as the nearest FP64 number (0 below its normal range)
+// f 2^X as the nearest FP64 number (0 below its normal range, infinite above it)
 __device__ __forceinline__ double to_double(long long f, int X) {
   unsigned long long u = f < 0 ? 0ull - (unsigned long long)f : (unsigned long long)f;
   const int n = __clzll((long long)u);
   const int e = 1023 + 63 - n + X;
   if (u == 0 || e < 1) return 0.0;
+  if (e > 2046) return __longlong_as_double(f < 0 ? (long long)0xfff0000000000000ull : 0x7ff0000000000000ll);
   u <<= n;
   unsigned long long v = u >> 11;
   const unsigned r = (unsigned)u & 0x7ffu;

@@ -31,6 +31,7 @@ __device__ __forceinline__ void block_sum_warp_totals(double wa, double wb, doub
     y = l < nw ? sb[l] : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
+      if (o >= nw) continue;  // lanes from nw on hold zeros
       x += __shfl_down_sync(0xffffffffu, x, o);
       y += __shfl_down_sync(0xffffffffu, y, o);
     }
@@ -108,8 +109,17 @@ __device__ __forceinline__ void grid_reduce_block_sums(double a, double b, doubl
     x += p.x;
     y += p.y;
   }
+  // warps without a pair hold zeros and skip their FP64 shuffle sums, which would
+  // share the FP64 pipe with the others' (a few us of a small lattice's gradient)
+  if ((threadIdx.x & ~31) < (int)gridDim.x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      x += __shfl_down_sync(0xffffffffu, x, o);
+      y += __shfl_down_sync(0xffffffffu, y, o);
+    }
+  }
   __syncthreads();  // the shared scratch of the block sum is reused
-  block_sum_mixed<double>(x, y, a, b);
+  block_sum_warp_totals(x, y, a, b);
   if (threadIdx.x == 0) {
     st->arrive = 0;
     finish_reduction(st, a, b, normF, normT, mode);
