@@ -909,7 +909,7 @@ struct lgf_batch_ctx {
   cudaStream_t main = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;        // source of exec (holds the members' loop conditions)
-  int lanes = 0;                      // parallel graph branches (0: one per member)
+  int lanes = -1;                     // parallel graph branches (0: one per member, -1: by the members' sizes)
   std::vector<int> exec_members;      // members captured in exec
   std::vector<long long> exec_launches;  // kernels per member per graph launch
   std::string err;
@@ -936,6 +936,22 @@ void drop_graph(lgf_batch b) {
   b->exec_members.clear();
 }
 
+// Lanes that a batch without set or tuned lanes runs on: as many as bring 2^20
+// sites together at the members' work-weighted size sum V^2 / sum V.  Small
+// lattices need many neighbours to fill the SMs (sixteen of 16^4: 16 lanes 6.7
+// ms, 8 6.7, 4 7.3, 2 8.6), large ones thrash L2 with more than two (two each of
+// 24^3 x 48, 32^3 x 8, 20^4 and 16^4: 2 lanes 12.9 ms, 4 14.1, 8 15.4).
+int default_lanes(lgf_batch b, const std::vector<int>& members) {
+  double v = 0.0, v2 = 0.0;
+  for (int i : members) {
+    const double n = (double)b->h[i]->V;
+    v += n;
+    v2 += n * n;
+  }
+  const double lanes = (double)(1 << 20) * v / v2;
+  return lanes < 1.5 ? 1 : lanes > (double)members.size() ? (int)members.size() : (int)(lanes + 0.5);
+}
+
 // One graph over the listed members: for each member a while node around one
 // captured iteration of its current engine, stopped by the member's own
 // on-device decision (lgf_reduce.cuh); the members' nodes run as parallel
@@ -945,7 +961,8 @@ int capture(lgf_batch b, const std::vector<int>& members, std::vector<unsigned l
   drop_graph(b);
   conds.assign(members.size(), 0);
   b->exec_launches.assign(members.size(), 0);
-  const int nl = (b->lanes <= 0 || b->lanes > (int)members.size()) ? (int)members.size() : b->lanes;
+  const int want = b->lanes < 0 ? default_lanes(b, members) : b->lanes;
+  const int nl = (want <= 0 || want > (int)members.size()) ? (int)members.size() : want;
   std::vector<size_t> order(members.size());
   for (size_t m = 0; m < order.size(); ++m) order[m] = m;
   std::stable_sort(order.begin(), order.end(),
