@@ -13,9 +13,9 @@
 // queue with DevState::unfit and the host runs the FP64 kernels on the
 // untouched FP64 links.
 //
-// 32^4, us per launch, FP64 kernels -> these: update 1570 -> 320, gradient
-// 395 -> 200, g 218 -> 158 (smaller CTAs); load and store of the pairs, once per queue, 180
-// each.
+// 32^4, us per launch, FP64 kernels -> these: update 1570 -> 307, gradient
+// 395 -> 118, g 218 -> 154 (smaller CTAs); load and store of the pairs, once
+// per queue, 180 each.
 #include "lgf_fx.cuh"
 #include "lgf_kernels.cuh"
 #include "lgf_reduce.cuh"
@@ -86,8 +86,16 @@ __device__ __forceinline__ void fx_add(fxacc& a, int h, float l) {
 // Delta from integer sums of the pairs, exact up to the FP32 sums of the low
 // parts; FP64 only from Delta on (theta, the traceless diagonal).  Grid-stride
 // over sites, so that the FP64 warp and block sums run once per thread.
+//
+// Bound by the loads in flight: all eight link matrices of a site are needed
+// for its sums.  Three CTAs of 128 an SM leave 168 registers a thread, which
+// hold them, and a grid of exactly those CTAs sweeps one contiguous region, so
+// that the links of x - mu are still in cache.  32^4: 118 us (671 MB of links
+// and Delta, 5.7 TB/s); eight CTAs of 128 at the compiler's own register count
+// 188, with two CTAs an SM 123, with five 187; 16^4 20.6 -> 18.5.
+constexpr int kGradFxCtas = 3;
 template <int NC>
-__global__ void __launch_bounds__(256) k_gradient_fx(const fx* __restrict__ U, cx<double>* __restrict__ D,
+__global__ void __launch_bounds__(128, kGradFxCtas) k_gradient_fx(const fx* __restrict__ U, cx<double>* __restrict__ D,
                                                      double2* __restrict__ partial, const Geom geo, DevState* st,
                                                      int mode, double normF, double normT) {
   pdl_wait();
@@ -326,7 +334,7 @@ cudaError_t launch_gradient_fx(int nc, const void* Ufx, void* D, double2* partia
                                int mode, cudaStream_t s) {
   const double nF = 1.0 / (12.0 * (double)geo.V), nT = 1.0 / (3.0 * (double)geo.V);
   const int thr = site_threads(geo.V);
-  const unsigned cap = 152 * 8, full = nblocks(geo.V, thr), nb = full < cap ? full : cap;
+  const unsigned cap = 152 * kGradFxCtas, full = nblocks(geo.V, thr), nb = full < cap ? full : cap;
   const auto u = static_cast<const fx*>(Ufx);
   auto d = static_cast<cx<double>*>(D);
   if (nc == 9) return launch_pdl(k_gradient_fx<9>, nb, thr, 0, s, u, d, partial, geo, st, mode, nF, nT);
