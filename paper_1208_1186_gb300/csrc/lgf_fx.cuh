@@ -111,6 +111,41 @@ __device__ __forceinline__ bool fx_from_double(double x, int& h, float& l) {
   return e <= 0;
 }
 
+// The row of three complex numbers as pairs relative to a power of two: the
+// largest exponent among the six numbers, or up to two more where the row's
+// norm would pass 1.97.  The norm of the result is then between 0.98 and 1.97.
+// False for a row that is not finite or not normal.
+__device__ __forceinline__ bool fx_row_from_double(const cx<double>* x, fx* r) {
+  unsigned long long b[6];
+  int top = 0;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    b[2 * j] = (unsigned long long)__double_as_longlong(x[j].re);
+    b[2 * j + 1] = (unsigned long long)__double_as_longlong(x[j].im);
+    top = max(top, max((int)(b[2 * j] >> 52) & 0x7ff, (int)(b[2 * j + 1] >> 52) & 0x7ff));
+  }
+  if (top == 0x7ff || top < 64) return false;
+  for (;; ++top) {  // each turn quarters n, which starts below 24
+    float n = 0.f;
+    int h[6];
+    float l[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      const int sh = 1 + top - (int)((b[j] >> 52) & 0x7ff);  // at least 64 where x is 0
+      const unsigned long long m = (b[j] << 11) | (1ull << 63);
+      long long f = sh < 64 ? (long long)(m >> (sh & 63)) : 0;
+      if ((long long)b[j] < 0) f = -f;
+      h[j] = (int)((long long)((unsigned long long)f + (1ull << 31)) >> 32);  // +-2^31 wraps: n is too large then
+      l[j] = __fmul_rn((float)(int)(unsigned)f, 0x1p-32f);
+      n = __fmaf_rn((float)h[j], (float)h[j], n);
+    }
+    if (n > 3.88f * 0x1p60f) continue;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) r[j] = {h[2 * j], l[2 * j], h[2 * j + 1], l[2 * j + 1]};
+    return true;
+  }
+}
+
 // f 2^-kScale as the nearest FP64 number, by bit manipulation
 template <int kScale>
 __device__ __forceinline__ double fx_scaled_to_double(long long f) {
@@ -133,6 +168,92 @@ __device__ __forceinline__ double fx_to_double(int h, float l) {
 // a sum of (h, l) pairs, in units of 2^-30 and at most 2^34 of them, as FP64
 __device__ __forceinline__ double fx_sum_to_double(const fxacc& a) {
   return fx_scaled_to_double<58>((a.h << 28) + __float2int_rn(__fmul_rn(a.l, 0x1p28f)));
+}
+
+// the squared norm of a row, below 4, in units of 2^-60
+__device__ __forceinline__ long long fx_norm2(const fx* r) {
+  fxacc n = {0, 0.f};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    fx_mac(n, fx_re(r[j]), fx_re(r[j]));
+    fx_mac(n, fx_im(r[j]), fx_im(r[j]));
+  }
+  // |n.l| < 2^33: to a multiple of 2^4, i.e. 2^-56
+  return n.h + ((long long)__float2int_rn(__fmul_rn(n.l, 0x1p-4f)) << 4);
+}
+
+// A row of squared norm n2 2^-60, above 1/4, to norm 1.  What the FP64 inverse
+// root leaves, some 2^-53, is a common factor of the row, an error that the
+// iterations add up: it is measured on the result and taken out to first order.
+__device__ __forceinline__ bool fx_normalize(fx* r, long long n2) {
+  fxr k;
+  const bool ok = fx_from_double(rsqrt(fx_scaled_to_double<60>(n2)), k.h, k.l);
+  k.f = (float)k.h;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    fxacc re = {0, 0.f}, im = {0, 0.f};
+    fx_mac(re, fx_re(r[j]), k);
+    fx_mac(im, fx_im(r[j]), k);
+    r[j] = fx_round(re, im);
+  }
+  const float c = __fmul_rn((float)(int)((1ll << 60) - fx_norm2(r)), 0x1p-61f);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    r[j].lr = __fmaf_rn((float)r[j].hr, c, r[j].lr);
+    r[j].li = __fmaf_rn((float)r[j].hi, c, r[j].li);
+  }
+  return ok;
+}
+
+// Rows 1 and 2 of a matrix to the orthonormal rows of its reunitarisation
+// (Gram-Schmidt, as reunitarize()).  A row's length cancels in its
+// normalisation, so each is taken relative to a power of two and the products
+// run on pairs; the two inverse square roots are FP64.  Where row 2 is nearly
+// parallel to row 1 its remainder is normalised in FP64.  False if the result
+// is not finite.
+__device__ __forceinline__ bool fx_reunitarize(const M3<double>& m, fx* r) {
+  bool ok = fx_row_from_double(m.e[0], r);
+  ok = ok && fx_row_from_double(m.e[1], r + 3);
+  if (!ok) return false;
+  ok = fx_normalize(r, fx_norm2(r));
+  fxacc pr = {0, 0.f}, pi = {0, 0.f};  // sum conj(r1_j) r2_j, at most the norm of row 2
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const fxr ur = fx_re(r[j]), ui = fx_im(r[j]), vr = fx_re(r[3 + j]), vi = fx_im(r[3 + j]);
+    fx_mac(pr, vr, ur);
+    fx_mac(pr, vi, ui);
+    fx_mac(pi, vi, ur);
+    fx_mac(pi, fx_neg(vr), ui);
+  }
+  const fx p = fx_neg(fx_round(pr, pi));
+  const fxr qr = fx_re(p), qi = fx_im(p);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const fxr ur = fx_re(r[j]), ui = fx_im(r[j]);
+    fxacc re = {(long long)r[3 + j].hr << 30, r[3 + j].lr * 0x1p30f};
+    fxacc im = {(long long)r[3 + j].hi << 30, r[3 + j].li * 0x1p30f};
+    fx_mac(re, qr, ur);
+    fx_mac(re, fx_neg(qi), ui);
+    fx_mac(im, qr, ui);
+    fx_mac(im, qi, ur);
+    r[3 + j] = fx_round(re, im);
+  }
+  const long long n2 = fx_norm2(r + 3);
+  if (n2 > 0x428ll << 48) return fx_normalize(r + 3, n2) && ok;  // 0.26
+  double w[6], n = 0.0;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    w[2 * j] = fx_to_double(r[3 + j].hr, r[3 + j].lr);
+    w[2 * j + 1] = fx_to_double(r[3 + j].hi, r[3 + j].li);
+    n = fma(w[2 * j], w[2 * j], fma(w[2 * j + 1], w[2 * j + 1], n));
+  }
+  n = rsqrt(n);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    ok = fx_from_double(w[2 * j] * n, r[3 + j].hr, r[3 + j].lr) && ok;
+    ok = fx_from_double(w[2 * j + 1] * n, r[3 + j].hi, r[3 + j].li) && ok;
+  }
+  return ok;
 }
 
 }  // namespace lgf
