@@ -13,7 +13,7 @@
 // queue with DevState::unfit and the host runs the FP64 kernels on the
 // untouched FP64 links.
 //
-// 32^4, us per launch, FP64 kernels -> these: update 1570 -> 307, gradient
+// 32^4, us per launch, FP64 kernels -> these: update 1570 -> 281, gradient
 // 395 -> 118, g 218 -> 54; load and store of the pairs, once per queue, 180
 // each.
 #include "lgf_fx.cuh"
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(128, kGradFxCtas) k_gradient_fx(const fx* __re
 // g from the accelerated gradient: 1 + alpha/2 Delta~ (or its exponential) in
 // FP64, the Gram-Schmidt on pairs (fx_reunitarize).  In FP64 throughout its 85
 // multiply-adds a site bound the kernel; on pairs 25 are left: 32^4 154 -> 54
-// us (4.0 TB/s), 16^4 12.8 -> 10.3.  Against 80-bit arithmetic, 28 iterations
+// us (4.0 TB/s), 16^4 16.9 -> 10.3.  Against 80-bit arithmetic, 28 iterations
 // of 8^4 leave links off by 3.2e-16 rms (FP64 kernels 4.7e-16; pairs with FP64
 // Gram-Schmidt 4.4e-16).  A non-finite g has no pair: the queue stops and is
 // reported as not finite.
@@ -229,18 +229,24 @@ __global__ void __launch_bounds__(128) k_accumulate_fx(cx<double>* G, const fx* 
   for (int q = 0; q < NC; ++q) G[q * V + s] = r.e[q / 3][q % 3];
 }
 
-// One thread per (site, direction), a block 32 sites x 4 directions (the warps
-// share g(x) through L1, and an 8^4 lattice fills 128 SMs).  w = g U row by
-// row, then the row of w g'^dag: 216 real multiply-adds per thread as 216
-// integer and 432 FP32 ones.
+// One thread per (site, direction): w = g U row by row, then the row of
+// w g'^dag: 216 real multiply-adds per thread as 216 integer and 432 FP32 ones.
+//
+// Bound by the links' round trip with few threads in flight, so a CTA is 64
+// sites of one direction: 1 KB runs in each of the planes, a direction that is
+// the same for the whole CTA (its neighbour stride is no select), g from L2 for
+// the four CTAs of the same sites that run side by side.  32^4 281 us (1.36 GB,
+// 4.8 TB/s); 32 sites x 4 directions in a CTA 307, 128 sites of one direction
+// 284, 256 377.  Six CTAs an SM hold all of NC = 9 in registers (eight: 299);
+// 12-real storage has room for eight (24^4 81 -> 74 us).
 template <int NC>
-__global__ void __launch_bounds__(128, 3) k_update_fx(fx* U, const fx* __restrict__ g, const Geom geo,
-                                                      const DevState* __restrict__ st) {
+__global__ void __launch_bounds__(64, NC == 9 ? 6 : 8) k_update_fx(fx* U, const fx* __restrict__ g, const Geom geo,
+                                                                   const DevState* __restrict__ st) {
   pdl_wait();
   if (st->done) return;
   const int V = (int)geo.V;
-  const int mu = threadIdx.x >> 5;
-  const int s = blockIdx.x * 32 + (threadIdx.x & 31);
+  const int mu = blockIdx.x & 3;
+  const int s = (blockIdx.x >> 2) * 64 + threadIdx.x;
   if (s >= V) return;
   int c[4];
   site_coords_r(geo, s, c);
@@ -356,8 +362,8 @@ cudaError_t launch_build_g_fx(int nc, const void* D, void* g, int64_t V, double 
 cudaError_t launch_update_fx(int nc, void* Ufx, const void* g, const Geom& geo, const DevState* st, cudaStream_t s) {
   auto u = static_cast<fx*>(Ufx);
   const auto gp = static_cast<const fx*>(g);
-  if (nc == 9) return launch_pdl(k_update_fx<9>, nblocks(geo.V, 32), 128, 0, s, u, gp, geo, st);
-  return launch_pdl(k_update_fx<6>, nblocks(geo.V, 32), 128, 0, s, u, gp, geo, st);
+  if (nc == 9) return launch_pdl(k_update_fx<9>, 4 * nblocks(geo.V, 64), 64, 0, s, u, gp, geo, st);
+  return launch_pdl(k_update_fx<6>, 4 * nblocks(geo.V, 64), 64, 0, s, u, gp, geo, st);
 }
 
 cudaError_t launch_accumulate_fx(int nc, void* G, const void* g, int64_t V, const DevState* st, cudaStream_t s) {
