@@ -81,10 +81,12 @@ enum lgf_param {
                             default 0: g is stored in FP32, so FP64 arithmetic
                             would be rounded away on the store)                */
   LGF_FFT_PIPELINE = 5,  /* FFT pipeline: 0 (default) automatic -- register
-                            planes (x-y + z-t passes) where instantiated, else
-                            per-axis register passes, else shared-memory
-                            Stockham planes; 1 Stockham planes; 2 per-axis
-                            passes; 3 register planes (1 where not available) */
+                            planes (x-y + z-t passes) of compiled-in extents
+                            where instantiated, else planes of any extents;
+                            1 planes of any extents; 2 per-axis passes; 3
+                            register planes (1 where not available).  Lines of
+                            an FP64 handle of up to 32 run in 64-bit block
+                            floating point in 1 and 3                        */
   LGF_TAIL_MODE = 7,     /* mixed precision: 0 (default) finishes with the
                             defect-correction tail when the FP32 phase reached
                             theta < 1e-8: FP32 acceleration and step, g = 1 +
@@ -321,11 +323,13 @@ int lgf_batch_fix(lgf_batch b, double theta_tol, int max_iter, int* iters_out, i
 /* Text of the last error of a batch call. */
 const char* lgf_batch_last_error(lgf_batch b);
 
-/* Parallel branches of the batch's graphs: 0 (the default) gives every member
- * its own branch; n > 0 spreads the members over n lanes (largest first, each
- * onto the lane with the fewest sites so far), a lane running its members'
- * iteration blocks one after another.  Fewer lanes keep fewer packed
- * gradients competing for L2.  Not part of the paper's method. */
+/* Parallel branches of the batch's graphs: 0 gives every member its own
+ * branch; n > 0 spreads the members over n lanes (largest first, each onto the
+ * lane with the fewest sites so far), a lane running its members' iteration
+ * blocks one after another.  A batch on which neither this nor the autotuner
+ * was called takes as many lanes as hold about a million sites together.  Fewer
+ * lanes keep fewer packed gradients competing for L2.  Not part of the paper's
+ * method. */
 int lgf_batch_set_lanes(lgf_batch b, int lanes);
 
 /* Lane autotuner: times one graph launch of reps iterations of every member
@@ -338,7 +342,7 @@ int lgf_batch_autotune(lgf_batch b, int reps, int* lanes_out);
  * the handle's engines, reps Fourier accelerations each, and use the fastest
  * from now on (unless LGF_FFT_PIPELINE forces a pipeline).  The schedules
  * are the pipelines (x-y/z-t register planes, per-axis register passes,
- * shared-memory Stockham planes) and, for the register planes, the x-run
+ * planes of any extents) and, for the register planes, the x-run
  * width of the z-t tiles (4 or 8 FP32 complex numbers, 2 or 4 FP64) and
  * the radix order of the z and t transforms (0: radix 4 first, 32 = 4 4 2;
  * 1: the same factors reversed, 32 = 2 4 4; FP32 only, where the stages
@@ -350,7 +354,7 @@ int lgf_batch_autotune(lgf_batch b, int reps, int* lanes_out);
  * lattice shape) for the process; if the environment variable
  * LGF_TUNE_CACHE names a file, the cache is written there (JSON) after each
  * tuning.  *chosen (may be NULL) receives the pipeline of the engine that
- * iterates first (1 Stockham planes, 2 axis passes, 3 register planes).
+ * iterates first (1 planes of any extents, 2 axis passes, 3 register planes).
  * Overwrites the gradient scratch only; the links are untouched.  Tile
  * widths give bit-identical results; radix orders round differently in
  * FP32 (the fix still ends at the same F to the FP64 tail's accuracy).

@@ -158,7 +158,7 @@ class GaugeFixer:
     def autotune(self, reps: int = 10) -> int:
         """Time the FFT schedules that apply to this lattice (pipelines, z-t
         tile widths, radix orders) and use the fastest; returns the pipeline
-        (1 Stockham planes, 2 axis passes, 3 register planes)."""
+        (1 planes of any extents, 2 axis passes, 3 register planes)."""
         ch = ctypes.c_int(0)
         _lib.check(self.lib.lgf_autotune(self.h, int(reps), ctypes.byref(ch)), "lgf_autotune", self.h)
         return ch.value
@@ -222,7 +222,8 @@ class GaugeBatch:
             raise LgfError(st, where, self.lib.lgf_batch_last_error(self.b).decode())
 
     def set_lanes(self, lanes: int):
-        """Parallel graph branches: 0 one per member, n > 0 n lanes."""
+        """Parallel graph branches: 0 one per member, n > 0 n lanes (if
+        never set: by the members' sizes)."""
         self._check(self.lib.lgf_batch_set_lanes(self.b, int(lanes)), "lgf_batch_set_lanes")
 
     def autotune(self, reps: int = 4) -> int:

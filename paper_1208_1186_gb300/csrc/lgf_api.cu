@@ -6,7 +6,10 @@
 // chain
 //   gradient -> reduce -> fft_xy(fwd) -> fft_zt(fwd, scale, inv)
 //            -> fft_xy(inv) -> build_g -> update [-> accumulate G]
-// on the handle's stream.  The reduce kernel decides on the device whether
+// on the handle's stream.  A plain FP64 handle runs its iterations on a copy
+// of the links in fixed-point pairs (lgf_fx.cuh), made at the start of a queue
+// and written back at its end; the FP64 kernels take over for links that do
+// not fit the pairs and on handles without room for them.  The reduce kernel decides on the device whether
 // the update of its iteration is applied (theta < tol or max_iter reached
 // stop the queue); every later kernel reads that decision first, so lgf_fix
 // queues LGF_CHECK_EVERY iterations between host synchronisations and still
