@@ -85,3 +85,19 @@ def test_non_finite_links_are_still_reported(lgf, bad):
         with pytest.raises(lgf.LgfError) as e:
             gf.fix(1e-12, 10)
         assert e.value.status == lgf._lib.LGF_ERR_NONFINITE
+
+
+@pytest.mark.parametrize("dims,alpha", [((4, 6, 2, 5), 0.125), ((4, 6, 2, 5), 1e-12), ((2, 2, 2, 60), 0.125)])
+@pytest.mark.parametrize("dtype", ["f64", "f64_r12"])
+def test_gauge_step_of_random_links(lgf, dims, alpha, dtype):
+    """Rows of 1 + alpha/2 Delta~ of any length and angle (random links; a long
+    axis, whose slow modes are accelerated by up to 10^3): taken relative to one
+    or two powers of two more, row 2 close to row 1.  Delta~ is good to some
+    1e-15 of its largest entry, and Gram-Schmidt divides by the sine of the
+    rows' angle, which stays above 1e-3 on a few hundred sites."""
+    U = I.synthetic_config(dims, seed=6, link_scale=3.0)
+    ref = O.iterate(U, 1, alpha)
+    with lgf.GaugeFixer(dims, dtype, alpha=alpha) as gf:
+        gf.load_links(U)
+        gf.iterate(1)
+        assert np.max(np.abs(gf.store_links() - ref)) <= 3e-12
