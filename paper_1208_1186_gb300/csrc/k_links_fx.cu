@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(128, kGradFxCtas) k_gradient_fx(const fx* __re
 // g from the accelerated gradient: 1 + alpha/2 Delta~ (or its exponential) in
 // FP64, the Gram-Schmidt on pairs (fx_reunitarize).  In FP64 throughout its 85
 // multiply-adds a site bound the kernel; on pairs 25 are left: 32^4 154 -> 54
-// us (4.0 TB/s), 16^4 16.9 -> 10.3.  Against 80-bit arithmetic, 28 iterations
+// us (4.0 TB/s), 16^4 16.9 -> 10.3; with the exponential, which stays FP64 and
+// bounds it, 16^3 x 32 takes 75.  Against 80-bit arithmetic, 28 iterations
 // of 8^4 leave links off by 3.2e-16 rms (FP64 kernels 4.7e-16; pairs with FP64
 // Gram-Schmidt 4.4e-16).  A non-finite g has no pair: the queue stops and is
 // reported as not finite.
