@@ -115,6 +115,16 @@ cudaError_t fft_any_init(int smem) {
   return e;
 }
 
+cudaError_t zt_pair_init(int Lz, int Lt) {
+  switch (Lz) {
+#define LGF_CASE(N) \
+  case N: return zt_pair_init<N>(Lt);
+    LGF_PAIR_EXTENTS(LGF_CASE)
+#undef LGF_CASE
+    default: return cudaSuccess;
+  }
+}
+
 cudaError_t launch_fft_xy(int prec, const int L[4], void* D, int inverse, const DevState* st, cudaStream_t s) {
   if (prec == 4 && plane_xy_supported(L[0], L[1]))
     return launch_plane_xy(L[0], D, (int64_t)L[0] * L[1] * L[2] * L[3], L[2], L[3], inverse, st, s);

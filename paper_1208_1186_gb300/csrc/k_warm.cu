@@ -940,11 +940,14 @@ cudaError_t launch_signal(const void* D, int V, float coef, void* gc, cudaStream
 
 namespace {
 template <int CI, int GC, int LG, int LO>
+cudaError_t wgrad_init() {
+  return cudaFuncSetAttribute(k_wgrad_tc<CI, GC, LG, LO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              WgShape<CI, GC>::kSmem);
+}
+
+template <int CI, int GC, int LG, int LO>
 cudaError_t wgrad_launch(const void* x, const void* gy, float* gW, const Geom& geo, int* err, cudaStream_t s) {
   using S = WgShape<CI, GC>;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      k_wgrad_tc<CI, GC, LG, LO>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
-  if (attr != cudaSuccess) return attr;
   const int64_t rows = (int64_t)(geo.L[0] + 2) * (geo.L[1] + 2) * geo.L[2] * geo.L[3];
   const int nchunks = (int)((rows + kWgRows - 1) / kWgRows);
   // three dt groups fill the 152 SMs with 50 CTAs each (100 where two fit an
@@ -991,16 +994,23 @@ cudaError_t launch_pack_weights(const float* p, void* W1, void* W2, void* W3, fl
 }
 
 namespace {
+// shared memory of the longest x extent's stages; a launch asks for its own
+// extent's
+template <int K, int N>
+constexpr int conv_tc_smem_max() {
+  return kTcStages * tc_stage_bytes<K, N>(kMaxL);
+}
+
+template <int K, int N, int SIGN, bool FWD>
+cudaError_t conv_tc_init() {
+  static_assert(conv_tc_smem_max<K, N>() <= 227 * 1024, "the stages fit one CTA's shared memory");
+  return cudaFuncSetAttribute(k_conv_tc<K, N, SIGN, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              conv_tc_smem_max<K, N>());
+}
+
 template <int K, int N, int SIGN, bool FWD>
 cudaError_t conv_tc_launch(const void* act, const void* Wk, const float* bias, const void* mask, void* y, float* yf,
                            const Geom& geo, bool relu, int* err, cudaStream_t s) {
-  // the stages of the longest x extent fix the attribute once; a launch asks
-  // for its own extent's stages
-  constexpr int smem_max = kTcStages * tc_stage_bytes<K, N>(kMaxL);
-  static_assert(smem_max <= 227 * 1024, "the stages fit one CTA's shared memory");
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_conv_tc<K, N, SIGN, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-  if (attr != cudaSuccess) return attr;
   if (geo.L[0] > kMaxL || geo.L[1] > kMaxL) return cudaErrorInvalidValue;
   const int smem = kTcStages * tc_stage_bytes<K, N>(geo.L[0]);
   // 128 rows per CTA over the (z, t) planes padded by a halo in x and y
@@ -1029,6 +1039,20 @@ cudaError_t launch_conv_bwd_data_tc(int layer, const void* gy, const void* W, co
                                     const Geom& geo, int* err, cudaStream_t s) {
   if (layer == 3) return conv_tc_launch<kOutPad, kHid, -1, false>(gy, W, nullptr, a, gx, nullptr, geo, false, err, s);
   return conv_tc_launch<kHid, kHid, -1, false>(gy, W, nullptr, a, gx, nullptr, geo, false, err, s);
+}
+
+// the kernels' shared memory limits on the current device (at creation of a
+// network: a limit belongs to the device, not to the process)
+cudaError_t init() {
+  cudaError_t e = conv_tc_init<kFeat, kHid, +1, true>();
+  if (e == cudaSuccess) e = conv_tc_init<kHid, kHid, +1, true>();
+  if (e == cudaSuccess) e = conv_tc_init<kHid, kOutPad, +1, true>();
+  if (e == cudaSuccess) e = conv_tc_init<kOutPad, kHid, -1, false>();
+  if (e == cudaSuccess) e = conv_tc_init<kHid, kHid, -1, false>();
+  if (e == cudaSuccess) e = wgrad_init<kFeat, kHid / 8, kHid, kHid>();
+  if (e == cudaSuccess) e = wgrad_init<kHid, kHid / 8, kHid, kHid>();
+  if (e == cudaSuccess) e = wgrad_init<kHid, kOut / 8, kOutPad, kOut>();
+  return e;
 }
 
 }  // namespace warm

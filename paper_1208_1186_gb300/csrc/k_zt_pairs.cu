@@ -17,21 +17,36 @@ namespace {
 constexpr int pair_bx(int m) { return m <= 8 ? 8 : 4; }
 
 template <int LZ, int LT>
+cudaError_t pair_init() {
+  constexpr int BX = pair_bx(LZ > LT ? LZ : LT);
+  constexpr size_t sm = zt_smem_bytes<float, LZ, LT, BX>();
+  if constexpr (sm > 48 * 1024)
+    return cudaFuncSetAttribute(k_plane_zt<LZ, LT, BX, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  return cudaSuccess;
+}
+
+template <int LZ, int LT>
 cudaError_t pair_launch(void* D, int Lx, int Ly, const float* s2p, float c_over_V, const DevState* st,
                         cudaStream_t s) {
   constexpr int BX = pair_bx(LZ > LT ? LZ : LT);
   constexpr size_t sm = zt_smem_bytes<float, LZ, LT, BX>();
-  if constexpr (sm > 48 * 1024) {  // once per process
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        k_plane_zt<LZ, LT, BX, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (attr != cudaSuccess) return attr;
-  }
   dim3 grid((unsigned)((Lx * Ly + BX - 1) / BX), 4);
   return launch_pdl(k_plane_zt<LZ, LT, BX, 0>, grid, zt_threads<LZ, LT, BX>(), sm, s,
                     static_cast<cx<float>*>(D), Lx, Ly, s2p, c_over_V, st);
 }
 
 }  // namespace
+
+template <int LZ>
+cudaError_t zt_pair_init(int Lt) {
+  switch (Lt) {
+#define LGF_CASE(LT) \
+  case LT: return pair_init<LZ, LT>();
+    LGF_PAIR_EXTENTS(LGF_CASE)
+#undef LGF_CASE
+    default: return cudaSuccess;
+  }
+}
 
 template <int LZ>
 cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* s2p, float c_over_V, const DevState* st,
@@ -45,6 +60,7 @@ cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* s2p, fl
   }
 }
 
+template cudaError_t zt_pair_init<LGF_PAIR_Z>(int);
 template cudaError_t launch_zt_pair<LGF_PAIR_Z>(int, void*, int, int, const float*, float, const DevState*,
                                                 cudaStream_t);
 

@@ -1332,6 +1332,7 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
     return bail(LGF_ERR_ARG);
   }
   cudaError_t e = fft_any_init(smem_optin);
+  if (e == cudaSuccess && h->mixed) e = zt_pair_init(h->L[2], h->L[3]);
   if (e == cudaSuccess) e = axis_pass_init();
   if (e == cudaSuccess) e = plane_pipeline_init();
   if (e != cudaSuccess) {
@@ -2092,6 +2093,10 @@ int lgf_net_create(unsigned long long seed, lgf_net* out) {
   if (cudaGetDevice(&n->device) != cudaSuccess) {
     delete n;
     return nfail(nullptr, LGF_ERR_CUDA, "no CUDA device");
+  }
+  if (const cudaError_t e = warm::init(); e != cudaSuccess) {
+    delete n;
+    return nfail(nullptr, LGF_ERR_CUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
   }
   const size_t P = warm::kParams;
   n->p = static_cast<float*>(net_alloc(n, P * 4));

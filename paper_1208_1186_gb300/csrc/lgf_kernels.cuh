@@ -95,6 +95,11 @@ template <int LZ>
 cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* s2p, float c_over_V, const DevState* st,
                            cudaStream_t s);
 bool zt_pair_supported(int prec, int Lz, int Lt);
+// raises the shared memory limit of a pair's kernel on the current device, at
+// handle creation; for this pair alone, because touching a kernel loads it
+template <int LZ>
+cudaError_t zt_pair_init(int Lt);
+cudaError_t zt_pair_init(int Lz, int Lt);
 // kfac[s] = p2max / (V sum_a s2[a][x_a]), 0 at the origin; s2: [4][kMaxL]
 cudaError_t launch_kfac(const int L[4], const double* s2, double p2max, double* kfac, cudaStream_t s);
 
@@ -186,6 +191,7 @@ cudaError_t launch_tail_update(void* U64, const void* eps, const Geom& geo, cons
 // exp map, training signal, Adam
 namespace warm {
 constexpr int kParams = 81 * 48 * 32 + 32 + 81 * 32 * 32 + 32 + 81 * 32 * 8 + 8;
+cudaError_t init();
 cudaError_t launch_features(int nc, const void* U0, void* x, const Geom& geo, cudaStream_t s);
 cudaError_t launch_expmap(int nc, const float* c, int ldc, void* G, int V, cudaStream_t s);
 cudaError_t launch_signal(const void* D, int V, float coef, void* gc, cudaStream_t s);
