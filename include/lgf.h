@@ -427,7 +427,9 @@ int lgf_net_forward(lgf_net n, lgf_handle h, float* host_c);
  * backward, and (if lr > 0) one Adam step (beta 0.9/0.999).  *F_out (may be
  * NULL) receives F(U^{g0}) before the step; host_grad (may be NULL) receives
  * the parameter gradient of -F (layout of lgf_net_get_params).  Leaves the
- * handle's links untouched. */
+ * handle's links untouched.  LGF_ERR_TIMEOUT (a bounded wait inside a kernel
+ * expired) leaves the network as it was, so that the step can be repeated;
+ * host_grad is not valid then. */
 int lgf_net_train_step(lgf_net n, lgf_handle h, double lr, double* F_out, float* host_grad);
 
 /* Install the predicted g0 as the initial gauge transformation of h; call

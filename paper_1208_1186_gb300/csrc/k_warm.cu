@@ -846,10 +846,13 @@ __global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ gy, 
 }
 
 // Adam on the FP32 master parameters; bf16 copies of the weights refreshed.
+// Nothing moves if a convolution of the step gave up a wait (*err): g is not the
+// gradient then.
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                       int n, float lr, float b1, float b2, float c1, float c2, float eps) {
+                       int n, float lr, float b1, float b2, float c1, float c2, float eps,
+                       const int* __restrict__ err) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || *err != 0) return;
   const float gi = g[i];
   const float mi = b1 * m[i] + (1.f - b1) * gi;
   const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
@@ -980,8 +983,8 @@ cudaError_t launch_bias_grad(int layer, const void* gy, float* gb, int V, cudaSt
 }
 
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float c1,
-                        float c2, float eps, cudaStream_t s) {
-  k_adam<<<(n + 255) / 256, 256, 0, s>>>(p, g, m, v, n, lr, b1, b2, c1, c2, eps);
+                        float c2, float eps, const int* err, cudaStream_t s) {
+  k_adam<<<(n + 255) / 256, 256, 0, s>>>(p, g, m, v, n, lr, b1, b2, c1, c2, eps, err);
   return cudaPeekAtLastError();
 }
 

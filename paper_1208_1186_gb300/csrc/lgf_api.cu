@@ -2216,11 +2216,11 @@ int lgf_net_train_step(lgf_net n, lgf_handle h, double lr, double* F_out, float*
   h->launches += 13;
   if (host_grad) LGF_NCUDA(n, cudaMemcpyAsync(host_grad, n->g, P * 4, cudaMemcpyDeviceToHost, s));
   if (lr > 0.0) {
-    n->step += 1;
-    const double b1 = 0.9, b2 = 0.999;
-    const float c1 = (float)(1.0 / (1.0 - pow(b1, (double)n->step)));
-    const float c2 = (float)(1.0 / (1.0 - pow(b2, (double)n->step)));
-    LGF_NCUDA(n, warm::launch_adam(n->p, n->g, n->m, n->v, (int)P, (float)lr, (float)b1, (float)b2, c1, c2, 1e-12f, s));
+    const double b1 = 0.9, b2 = 0.999, step = (double)(n->step + 1);
+    const float c1 = (float)(1.0 / (1.0 - pow(b1, step)));
+    const float c2 = (float)(1.0 / (1.0 - pow(b2, step)));
+    LGF_NCUDA(n, warm::launch_adam(n->p, n->g, n->m, n->v, (int)P, (float)lr, (float)b1, (float)b2, c1, c2, 1e-12f,
+                                   n->tc_err, s));
     rc = net_pack(n, s);
     if (rc) return rc;
     h->launches += 2;
@@ -2229,6 +2229,7 @@ int lgf_net_train_step(lgf_net n, lgf_handle h, double lr, double* F_out, float*
   if (rc) return nfail(n, rc, h->err);
   rc = net_check_tc(n);
   if (rc) return rc;
+  if (lr > 0.0) n->step += 1;
   if (F_out) *F_out = h->st_host->F;
   return LGF_OK;
 }

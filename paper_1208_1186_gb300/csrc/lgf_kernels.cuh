@@ -200,7 +200,7 @@ cudaError_t launch_conv_bwd_weight(int layer, const void* x, const void* gy, flo
                                    cudaStream_t s);
 cudaError_t launch_bias_grad(int layer, const void* gy, float* gb, int V, cudaStream_t s);
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float c1,
-                        float c2, float eps, cudaStream_t s);
+                        float c2, float eps, const int* err, cudaStream_t s);  // *err set: no change
 cudaError_t launch_pack_weights(const float* p, void* W1, void* W2, void* W3, float* b1, float* b2, float* b3,
                                 void* Wt1, void* Wt2, void* Wt3, cudaStream_t s);
 // tcgen05 implicit-GEMM convolutions (forward and backward data); err[0] is
