@@ -452,6 +452,14 @@ int lgf_net_warm_start(lgf_net n, lgf_handle h);
 int lgf_net_conv(lgf_net n, int layer, int backward, const void* in, const void* mask, void* out, float* out_f32,
                  int Lx, int Ly, int Lz, int Lt, void* stream);
 
+/* The third direction of such a layer: its weight gradient gW [81][in][out]
+ * (FP32, device memory, overwritten; out = 32, 32, 8) from the layer's input in
+ * ([V][48], [V][32], [V][32]) and the gradient gy with respect to its output
+ * ([V][32], [V][32], [V][16]; of layer 3's channels the first 8).  In, gy and
+ * the rest as lgf_net_conv. */
+int lgf_net_conv_weight_grad(lgf_net n, int layer, const void* in, const void* gy, float* gW, int Lx, int Ly, int Lz,
+                             int Lt, void* stream);
+
 /* Poll budget of the waits inside the tensor-core convolutions that wait for
  * a pipeline stage's MMAs (default and upper bound 2^22 polls; polls < 0
  * restores the default).  With a budget of 0 every such wait expires at

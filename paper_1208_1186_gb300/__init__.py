@@ -321,6 +321,19 @@ class WarmStartNet:
                                           *[int(d) for d in dims], ctypes.c_void_p(st)), "lgf_net_conv")
         return out
 
+    def conv_weight_grad(self, layer: int, x, gy, dims):
+        """Weight gradient [81][in][out] (FP32 tensor) of one layer from its
+        device bf16 input x and output gradient gy (lgf_net_conv_weight_grad)."""
+        import torch
+        nin, nout = {1: (48, 32), 2: (32, 32), 3: (32, 8)}[layer]
+        gW = torch.empty((81, nin, nout), dtype=torch.float32, device=x.device)
+        st = torch.cuda.current_stream().cuda_stream
+        self._check(self.lib.lgf_net_conv_weight_grad(self.n, int(layer), ctypes.c_void_p(x.data_ptr()),
+                                                      ctypes.c_void_p(gy.data_ptr()), ctypes.c_void_p(gW.data_ptr()),
+                                                      *[int(d) for d in dims], ctypes.c_void_p(st)),
+                    "lgf_net_conv_weight_grad")
+        return gW
+
     def set_wait_budget(self, polls: int):
         """Poll budget of the convolutions' stage waits (lgf_net_set_wait_budget;
         negative: the default)."""

@@ -2246,6 +2246,21 @@ int lgf_net_warm_start(lgf_net n, lgf_handle h) {
   return net_check_tc(n);
 }
 
+// geometry of a caller's lattice; false for an extent outside [2, 64]
+static bool net_geometry(int Lx, int Ly, int Lz, int Lt, Geom* geo) {
+  const int Ls[4] = {Lx, Ly, Lz, Lt};
+  int64_t V = 1;
+  for (int a = 0; a < 4; ++a) {
+    if (Ls[a] < 2 || Ls[a] > kMaxL) return false;
+    geo->L[a] = Ls[a];
+    geo->stride[a] = V;
+    V *= Ls[a];
+  }
+  geo->V = V;
+  geom_init_rcp(*geo);
+  return true;
+}
+
 int lgf_net_conv(lgf_net n, int layer, int backward, const void* in, const void* mask, void* out, float* out_f32,
                  int Lx, int Ly, int Lz, int Lt, void* stream) {
   if (!n) return LGF_ERR_ARG;
@@ -2253,16 +2268,8 @@ int lgf_net_conv(lgf_net n, int layer, int backward, const void* in, const void*
     return nfail(n, LGF_ERR_ARG, "lgf_net_conv: layer 1..3 forward, 2..3 backward");
   if (!in || !out) return nfail(n, LGF_ERR_ARG, "lgf_net_conv: in and out must be device pointers");
   Geom geo{};
-  const int Ls[4] = {Lx, Ly, Lz, Lt};
-  int64_t V = 1;
-  for (int a = 0; a < 4; ++a) {
-    if (Ls[a] < 2 || Ls[a] > kMaxL) return nfail(n, LGF_ERR_ARG, "lgf_net_conv: each extent must be in [2, 64]");
-    geo.L[a] = Ls[a];
-    geo.stride[a] = V;
-    V *= Ls[a];
-  }
-  geo.V = V;
-  geom_init_rcp(geo);
+  if (!net_geometry(Lx, Ly, Lz, Lt, &geo))
+    return nfail(n, LGF_ERR_ARG, "lgf_net_conv: each extent must be in [2, 64]");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   void* const Wt[3] = {n->Wt1, n->Wt2, n->Wt3};
   void* const W[3] = {n->W1, n->W2, n->W3};
@@ -2271,6 +2278,22 @@ int lgf_net_conv(lgf_net n, int layer, int backward, const void* in, const void*
     LGF_NCUDA(n, warm::launch_conv_fwd_tc(layer, in, Wt[layer - 1], b[layer - 1], out, out_f32, geo, n->tc_err, s));
   else
     LGF_NCUDA(n, warm::launch_conv_bwd_data_tc(layer, in, W[layer - 1], mask, out, geo, n->tc_err, s));
+  LGF_NCUDA(n, cudaStreamSynchronize(s));
+  return net_check_tc(n);
+}
+
+int lgf_net_conv_weight_grad(lgf_net n, int layer, const void* in, const void* gy, float* gW, int Lx, int Ly, int Lz,
+                             int Lt, void* stream) {
+  if (!n) return LGF_ERR_ARG;
+  if (layer < 1 || layer > 3) return nfail(n, LGF_ERR_ARG, "lgf_net_conv_weight_grad: layer 1..3");
+  if (!in || !gy || !gW) return nfail(n, LGF_ERR_ARG, "lgf_net_conv_weight_grad: in, gy and gW must be device pointers");
+  Geom geo{};
+  if (!net_geometry(Lx, Ly, Lz, Lt, &geo))
+    return nfail(n, LGF_ERR_ARG, "lgf_net_conv_weight_grad: each extent must be in [2, 64]");
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const int count[3] = {kW1, kW2, kW3};
+  LGF_NCUDA(n, cudaMemsetAsync(gW, 0, (size_t)count[layer - 1] * sizeof(float), s));
+  LGF_NCUDA(n, warm::launch_conv_bwd_weight(layer, in, gy, gW, geo, n->tc_err, s));
   LGF_NCUDA(n, cudaStreamSynchronize(s));
   return net_check_tc(n);
 }
