@@ -2038,22 +2038,32 @@ int lgf_batch_autotune(lgf_batch b, int reps, int* lanes_out) {
     return bfail(b, LGF_ERR_CUDA, "event creation failed");
   }
   const int cands[] = {1, 2, 4, 8, 16, 0};
-  int best = 0, rc = LGF_OK;
+  int best = 0;
   float best_ms = INFINITY;
   const int saved = b->lanes;
+  // the members run as run_members runs them: plain FP64 ones on their links in
+  // fixed-point pairs if they fit (the updates, which are unitary, keep them so)
+  std::vector<unsigned long long> conds(all.size(), 0);
+  for (int i : all) b->h[i]->fx = b->h[i]->Ufx != nullptr;
+  int rc = reset_members(b, all, tol, cap, nostall, conds);
+  if (!rc) rc = queue_fx_members(b, all, queue_fx_load);
+  if (!rc) rc = read_members(b, all);
+  for (int i : all) b->h[i]->fx = b->h[i]->fx && !b->h[i]->st_host->unfit;
   for (int c : cands) {
+    if (rc) break;
     if (c > n) continue;
     b->lanes = c;
-    std::vector<unsigned long long> conds;
     rc = capture(b, all, conds);
     if (rc) break;
     for (int pass = 0; pass < 2 && !rc; ++pass) {  // a warm-up launch, then the timed one
       rc = reset_members(b, all, tol, cap, nostall, conds);
+      if (!rc) rc = queue_fx_members(b, all, queue_fx_load);
       if (rc) break;
       cudaEventRecord(e0, b->main);
       if (cudaGraphLaunch(b->exec, b->main) != cudaSuccess) rc = bfail(b, LGF_ERR_CUDA, "graph launch failed");
       cudaEventRecord(e1, b->main);
-      if (!rc && cudaEventSynchronize(e1) != cudaSuccess) rc = bfail(b, LGF_ERR_CUDA, "graph launch failed");
+      if (!rc) rc = queue_fx_members(b, all, queue_fx_store);
+      if (!rc && cudaStreamSynchronize(b->main) != cudaSuccess) rc = bfail(b, LGF_ERR_CUDA, "graph launch failed");
       for (int i : all) b->h[i]->total_updates += reps;  // the tuning updates are applied
     }
     if (rc) break;
@@ -2067,6 +2077,7 @@ int lgf_batch_autotune(lgf_batch b, int reps, int* lanes_out) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   drop_graph(b);
+  for (int i : all) b->h[i]->fx = false;
   if (rc) {
     b->lanes = saved;
     return rc;
