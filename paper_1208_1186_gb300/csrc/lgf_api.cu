@@ -693,8 +693,7 @@ int run_queue(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_chec
       *unfit = true;
       return LGF_OK;
     }
-    if (s.nonfinite) return fail(h, LGF_ERR_NONFINITE, "F or theta is not finite (non-SU(3) or NaN input links?)");
-    if (s.done || queued >= (long long)max_iter + 1) break;
+    if (s.nonfinite || s.done || queued >= (long long)max_iter + 1) break;
     // predict the iterations still needed from the last interval
     int next = h->check_every;
     const int dn = s.iters - prev_iters;
@@ -713,6 +712,7 @@ int run_queue(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_chec
   if (!rc && h->fx) rc = sync_state(h);
   if (rc) return rc;
   const DevState& s = *h->st_host;
+  if (s.nonfinite) return fail(h, LGF_ERR_NONFINITE, "F or theta is not finite (non-SU(3) or NaN input links?)");
   *done_iters = s.iters;
   h->hist_n = s.iters + 1 < h->hist_cap ? s.iters + 1 : h->hist_cap;
   *converged = s.theta < tol;
