@@ -168,6 +168,14 @@ constexpr bool kDeviceLoops = true;
 // graph (sixteen of 16^4: 6.7 ms, with two 7.1).
 constexpr int kLoopUnroll = 2;
 
+// Smallest tolerance that plain FP64 iterations on fixed-point pairs are asked
+// to reach.  Their absolute resolution stops theta at 1e-31 to 2e-31 on every
+// lattice measured (8^4 to 32^4, 4^3 x 64, 12-real); FP64 links get to 6e-33, and
+// below 1e-40 on fields near the identity, whose small entries keep their
+// relative precision.  Smaller tolerances run on the FP64 kernels.
+constexpr double kFxTheta = 1e-28;
+bool fx_reaches(double tol) { return tol < 0.0 || tol >= kFxTheta; }
+
 int fail(lgf_handle h, int code, const std::string& msg) {
   if (h)
     h->err = msg;
@@ -720,11 +728,12 @@ int run_queue(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_chec
 }
 
 // run_queue on the fixed-point pairs of a plain FP64 handle where its links
-// fit them, else on the engine's own links.
+// fit them and the tolerance is within their reach, else on the engine's own
+// links.
 int run_fix(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
             int* done_iters, bool* converged) {
   bool unfit = false;
-  if (h->Ufx) {
+  if (h->Ufx && fx_reaches(tol)) {
     h->fx = true;
     const int rc = run_queue(h, e, tol, max_iter, stall_check, done_iters, converged, &unfit);
     h->fx = false;
@@ -1082,12 +1091,14 @@ int queue_fx_members(lgf_batch b, const std::vector<int>& members, int (*queue)(
 // budget, or -- with stall_check -- theta below 1e-6 no longer halving within
 // 8 updates): one launch of the batch graph, every member looping on the
 // device until its own stop decision.
-// Plain FP64 members run on their links in fixed-point pairs (allow_fx);
-// those whose links do not fit run again on their FP64 links.
+// Plain FP64 members run on their links in fixed-point pairs (allow_fx) where
+// their tolerance allows; those whose links do not fit run again on their FP64
+// links.
 int run_members(lgf_batch b, const std::vector<int>& members, const std::vector<double>& tol,
                 const std::vector<int>& max_iter, const std::vector<char>& stall_check, bool allow_fx = true) {
   if (members.empty()) return LGF_OK;
-  for (int i : members) b->h[i]->fx = allow_fx && b->h[i]->Ufx;
+  for (size_t m = 0; m < members.size(); ++m)
+    b->h[members[m]]->fx = allow_fx && b->h[members[m]]->Ufx && fx_reaches(tol[m]);
   auto leave_fx = [&](int rc) {
     for (int i : members) b->h[i]->fx = false;
     return rc;
