@@ -127,7 +127,11 @@ enum lgf_param {
 
 /* Device allocator hooks.  alloc returns a device pointer (NULL on failure);
  * free releases it.  Passing NULL for both restores cudaMalloc/cudaFree.
- * Process-wide; affects handles created afterwards. */
+ * Process-wide; affects handles created afterwards.  One buffer of an FP64
+ * handle is optional (its working copy of the links): when alloc returns NULL
+ * for another buffer, of any handle or network of the device, the library
+ * frees such a copy, possibly of a handle of another thread that is in no call,
+ * and asks again. */
 typedef void* (*lgf_alloc_fn)(size_t bytes, int device, void* stream, void* user);
 typedef void (*lgf_free_fn)(void* ptr, size_t bytes, int device, void* stream, void* user);
 int lgf_set_allocator(lgf_alloc_fn alloc, lgf_free_fn free_fn, void* user);
@@ -138,7 +142,9 @@ int lgf_set_allocator(lgf_alloc_fn alloc, lgf_free_fn free_fn, void* user);
  * passed by value to every kernel); Sec. 3.1: single or double precision,
  * 18-real or 12-real storage, the dtype choices here.  Each extent must be in [2, 64] and a
  * product of 2, 3 and 5 (the radices of the on-chip FFT); dtype is an
- * lgf_dtype.  Allocates all device buffers.  On failure *out is NULL and
+ * lgf_dtype.  Allocates all device buffers; an FP64 handle also takes a working
+ * copy of its links, for iterations about three times faster, if there is room,
+ * and gives it up for good when an allocation of the library finds none.  On failure *out is NULL and
  * lgf_last_error(NULL) describes the cause. */
 int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out);
 

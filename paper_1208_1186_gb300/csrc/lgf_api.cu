@@ -20,6 +20,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <condition_variable>
 #include <map>
 #include <mutex>
 #include <new>
@@ -105,7 +106,9 @@ struct lgf_ctx {
   bool g_valid = false;       // G (with the tail's Gh, Gl and eta) describes the current links
   int tail_mode = 0;          // defect-correction tail when the FP32 phase reached 1e-8, with links in
                               // double-float (0) or FP64 (2); 1: plain FP64
-  void* Ufx = nullptr;        // plain FP64 handles: the links in fixed-point pairs while a queue runs
+  void* Ufx = nullptr;        // plain FP64 handles: the links in fixed-point pairs while a queue runs (may be
+                              // null: see FxUse)
+  int fx_uses = 0;            // calls running on Ufx; under g_fx_mutex
   bool fx = false;            // ... the queue being built or captured runs on them
   bool defect = false;        // the FP64 engine runs the defect-correction tail
   bool df = false;            // ... on the double-float links in Udf (converted back at the end)
@@ -222,27 +225,112 @@ cudaError_t prof_end(lgf_handle h) {
     (h)->launches += 1;                                       \
   } while (0)
 
-void* dev_alloc(lgf_handle h, size_t bytes) {
-  if (bytes == 0) bytes = 16;
+// the allocator's memory, or null
+void* raw_alloc(size_t bytes, int device, cudaStream_t stream) {
   void* p = nullptr;
   if (g_alloc.alloc) {
-    p = g_alloc.alloc(bytes, h->device, (void*)h->stream, g_alloc.user);
+    p = g_alloc.alloc(bytes, device, (void*)stream, g_alloc.user);
   } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
     (void)cudaGetLastError();
     p = nullptr;
   }
+  return p;
+}
+
+void raw_free(void* p, size_t bytes, int device, cudaStream_t stream) {
+  if (g_alloc.free_fn)
+    g_alloc.free_fn(p, bytes, device, (void*)stream, g_alloc.user);
+  else
+    cudaFree(p);
+}
+
+// The pairs of plain FP64 handles (Ufx) are optional memory: a handle works
+// without them, on its FP64 kernels.  So an allocation of this library that finds
+// no room takes them back, from any handle of the device whose pairs no call is
+// using (a call that is using them is waited for), and tries again; what fitted
+// the device before there were pairs still does.  A handle whose pairs were taken
+// goes on without.
+std::mutex g_fx_mutex;
+std::condition_variable g_fx_idle;
+std::vector<lgf_handle> g_fx_holders;  // handles with Ufx
+
+size_t fx_bytes(lgf_handle h) { return (size_t)4 * h->e64.nc * h->V * sizeof(cx<double>); }
+
+// While one lives, a handle's pairs stay.  (No allocation is made meanwhile.)
+struct FxUse {
+  std::vector<lgf_handle> used;
+  explicit FxUse(lgf_handle h) : used{h} { add(+1); }
+  FxUse(const std::vector<lgf_handle>& all, const std::vector<int>& members) {
+    for (int i : members) used.push_back(all[i]);
+    add(+1);
+  }
+  FxUse(const FxUse&) = delete;
+  ~FxUse() { add(-1); }
+
+ private:
+  void add(int n) {
+    std::lock_guard<std::mutex> lock(g_fx_mutex);
+    for (lgf_handle h : used) h->fx_uses += n;
+    if (n < 0) g_fx_idle.notify_all();
+  }
+};
+
+// Takes h's pairs out of the handle (under g_fx_mutex; a loop captured on them is
+// not launched without them).  They are freed after the lock is released: an
+// allocator's callback may run arbitrary host code, the end of another handle
+// among it.
+void* detach_pairs(lgf_handle h) {
+  g_fx_holders.erase(std::find(g_fx_holders.begin(), g_fx_holders.end(), h));
+  void* p = h->Ufx;
+  h->Ufx = nullptr;
+  return p;
+}
+
+// one handle's pairs back to the allocator; false if no handle of the device holds any
+bool give_up_pairs(int device) {
+  std::unique_lock<std::mutex> lock(g_fx_mutex);
+  for (;;) {
+    bool busy = false;
+    for (lgf_handle h : g_fx_holders) {
+      if (h->device != device) continue;
+      if (h->fx_uses == 0) {  // its calls have waited for their work
+        const size_t bytes = fx_bytes(h);
+        const cudaStream_t stream = h->stream;
+        void* p = detach_pairs(h);
+        lock.unlock();
+        raw_free(p, bytes, device, stream);
+        return true;
+      }
+      busy = true;
+    }
+    if (!busy) return false;
+    g_fx_idle.wait(lock);
+  }
+}
+
+// memory that a handle or network needs
+void* required_alloc(size_t bytes, int device, cudaStream_t stream) {
+  void* p = raw_alloc(bytes, device, stream);
+  while (!p && give_up_pairs(device)) p = raw_alloc(bytes, device, stream);
+  return p;
+}
+
+void* dev_alloc(lgf_handle h, size_t bytes) {
+  if (bytes == 0) bytes = 16;
+  void* p = required_alloc(bytes, h->device, h->stream);
   if (p) h->allocs.push_back({p, bytes});
   return p;
 }
 
 void dev_free_all(lgf_handle h) {
-  for (auto& a : h->allocs) {
-    if (g_alloc.free_fn)
-      g_alloc.free_fn(a.p, a.n, h->device, (void*)h->stream, g_alloc.user);
-    else
-      cudaFree(a.p);
-  }
+  for (auto& a : h->allocs) raw_free(a.p, a.n, h->device, h->stream);
   h->allocs.clear();
+  void* p = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_fx_mutex);
+    if (h->Ufx) p = detach_pairs(h);
+  }
+  if (p) raw_free(p, fx_bytes(h), h->device, h->stream);
 }
 
 int alloc_engine(lgf_handle h, Engine& e) {
@@ -733,10 +821,12 @@ int run_queue(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_chec
 int run_fix(lgf_handle h, Engine& e, double tol, int max_iter, bool stall_check,
             int* done_iters, bool* converged) {
   bool unfit = false;
+  const FxUse use(h);
   if (h->Ufx && fx_reaches(tol)) {
     h->fx = true;
     const int rc = run_queue(h, e, tol, max_iter, stall_check, done_iters, converged, &unfit);
     h->fx = false;
+    if (rc) cudaStreamSynchronize(h->stream);  // nothing still runs on the pairs
     if (rc || !unfit) return rc;
   }
   return run_queue(h, e, tol, max_iter, stall_check, done_iters, converged, &unfit);
@@ -1097,10 +1187,12 @@ int queue_fx_members(lgf_batch b, const std::vector<int>& members, int (*queue)(
 int run_members(lgf_batch b, const std::vector<int>& members, const std::vector<double>& tol,
                 const std::vector<int>& max_iter, const std::vector<char>& stall_check, bool allow_fx = true) {
   if (members.empty()) return LGF_OK;
+  const FxUse use(b->h, members);
   for (size_t m = 0; m < members.size(); ++m)
     b->h[members[m]]->fx = allow_fx && b->h[members[m]]->Ufx && fx_reaches(tol[m]);
   auto leave_fx = [&](int rc) {
     for (int i : members) b->h[i]->fx = false;
+    if (rc) cudaStreamSynchronize(b->main);  // nothing still runs on the pairs
     return rc;
   };
   std::vector<unsigned long long> conds;
@@ -1186,13 +1278,7 @@ int nfail(lgf_net n, int code, const std::string& msg) {
   } while (0)
 
 void* net_alloc(lgf_net n, size_t bytes) {
-  void* q = nullptr;
-  if (g_alloc.alloc) {
-    q = g_alloc.alloc(bytes, n->device, nullptr, g_alloc.user);
-  } else if (cudaMalloc(&q, bytes) != cudaSuccess) {
-    (void)cudaGetLastError();
-    q = nullptr;
-  }
+  void* q = required_alloc(bytes, n->device, nullptr);
   if (q) n->allocs.push_back({q, bytes});
   return q;
 }
@@ -1200,10 +1286,7 @@ void* net_alloc(lgf_net n, size_t bytes) {
 void net_free(lgf_net n, void* q) {
   for (size_t i = 0; i < n->allocs.size(); ++i)
     if (n->allocs[i].first == q) {
-      if (g_alloc.free_fn)
-        g_alloc.free_fn(q, n->allocs[i].second, n->device, nullptr, g_alloc.user);
-      else
-        cudaFree(q);
+      raw_free(q, n->allocs[i].second, n->device, nullptr);
       n->allocs.erase(n->allocs.begin() + i);
       return;
     }
@@ -1359,8 +1442,6 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
   }
   if (rc) return bail(rc);
   h->cur = h->mixed ? &h->e32 : &h->e64;
-  // without it (no memory left) the handle iterates on its FP64 links
-  if (!h->mixed) h->Ufx = dev_alloc(h, (size_t)4 * h->e64.nc * V * 16);
   if (h->mixed) {
     h->G = dev_alloc(h, (size_t)h->e32.nc * V * h->e32.cbytes());
     h->Uorig = static_cast<double*>(dev_alloc(h, (size_t)4 * 9 * V * 16));
@@ -1386,6 +1467,11 @@ int lgf_create(int Lx, int Ly, int Lz, int Lt, int dtype, lgf_handle* out) {
   if (reset_state(h, -1.0, 0, false) || cudaStreamSynchronize(h->stream) != cudaSuccess) {
     h->err = "state initialisation failed";
     return bail(LGF_ERR_CUDA);
+  }
+  // last: what is left after everything needed
+  if (!h->mixed && (h->Ufx = raw_alloc(fx_bytes(h), h->device, h->stream)) != nullptr) {
+    std::lock_guard<std::mutex> lock(g_fx_mutex);
+    g_fx_holders.push_back(h);
   }
   *out = h;
   return LGF_OK;
@@ -1594,6 +1680,7 @@ int lgf_iterate(lgf_handle h, int n) {
   if (!h->loaded) return fail(h, LGF_ERR_ARG, "no links loaded");
   // first on the fixed-point pairs of a plain FP64 handle, then, if its links
   // do not fit them (nothing was done), on the engine's own links
+  const FxUse use(h);
   int rc = LGF_OK;
   for (int pass = h->Ufx ? 0 : 1; pass < 2 && !rc; ++pass) {
     h->fx = pass == 0;
@@ -1605,6 +1692,7 @@ int lgf_iterate(lgf_handle h, int n) {
     if (!rc) rc = sync_state(h);
     if (!rc && !h->st_host->unfit) break;
   }
+  if (rc) cudaStreamSynchronize(h->stream);  // nothing still runs on the pairs
   if (rc) return rc;
   if (h->st_host->nonfinite) return fail(h, LGF_ERR_NONFINITE, "F or theta is not finite");
   h->total_updates += h->st_host->iters;
@@ -2055,6 +2143,7 @@ int lgf_batch_autotune(lgf_batch b, int reps, int* lanes_out) {
   // the members run as run_members runs them: plain FP64 ones on their links in
   // fixed-point pairs if they fit (the updates, which are unitary, keep them so)
   std::vector<unsigned long long> conds(all.size(), 0);
+  const FxUse use(b->h, all);
   for (int i : all) b->h[i]->fx = b->h[i]->Ufx != nullptr;
   int rc = reset_members(b, all, tol, cap, nostall, conds);
   if (!rc) rc = queue_fx_members(b, all, queue_fx_load);
@@ -2087,8 +2176,9 @@ int lgf_batch_autotune(lgf_batch b, int reps, int* lanes_out) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  drop_graph(b);
   for (int i : all) b->h[i]->fx = false;
+  if (rc) cudaStreamSynchronize(b->main);  // nothing still runs on the pairs
+  drop_graph(b);
   if (rc) {
     b->lanes = saved;
     return rc;
