@@ -17,7 +17,7 @@
 #pragma once
 
 #include "fft_any_geom.cuh"
-#include "fft_reg.cuh"
+#include "zt_plane.cuh"
 
 namespace lgf {
 namespace anyfft {
@@ -75,9 +75,9 @@ __device__ __noinline__ void x_line(cx<T>* row) {
 }
 
 // forward t, times the acceleration factor, inverse t.  FP32: c / (a + s2t),
-// 0 at the origin; FP64: the table at kl, step apart.
+// rounded once, 0 at the origin; FP64: the table at kl, step apart.
 template <int L, class T>
-__device__ __noinline__ void t_line(cx<T>* line, int PT, float a, bool origin, float c_over_V, const T* kl, int step) {
+__device__ __noinline__ void t_line(cx<T>* line, int PT, df a, bool origin, df c, const T* kl, int step) {
   cx<T> v[L];
   cx<T>* p = line;
 #pragma unroll
@@ -89,10 +89,7 @@ __device__ __noinline__ void t_line(cx<T>* line, int PT, float a, bool origin, f
   if constexpr (sizeof(T) == 4) {
     regfft::static_for<0, L>([&](auto pc) {
       constexpr int i = decltype(pc)::value;
-      constexpr float s2t = (float)regfft::MomentumSq<L, i>::value;
-      float kf = c_over_V * rcp_approx(a + s2t);
-      if (i == 0 && origin) kf = 0.0f;
-      v[i] = scale(v[i], (T)kf);
+      v[i] = scale(v[i], (T)(i == 0 && origin ? 0.0f : factor_rounded<L, i>(c, a)));
     });
   } else {
 #pragma unroll
@@ -175,8 +172,8 @@ constexpr int zt_min_blocks() {
 // columns of a (z, t) site are contiguous, and a run may cross from one y to
 // the next.  z lines come from global memory into registers, go to the t lines
 // through shared memory, and are stored from registers after the inverse.
-// FP32: the factor from s2p[axis][position] and c_over_V as in k_plane_zt;
-// FP64: the per-site table kfac.
+// FP32: the factor from s2p and c_over_V as in k_plane_zt (EXACT); FP64: the
+// per-site table kfac.
 template <class T, int kMaxLen>
 __global__ void __launch_bounds__((zt_max_threads<T, kMaxLen>()), (zt_min_blocks<T, kMaxLen>()))
     k_any_zt(cx<T>* __restrict__ D, const ZtGeom g, const T* __restrict__ kfac, const float* __restrict__ s2p,
@@ -197,10 +194,13 @@ __global__ void __launch_bounds__((zt_max_threads<T, kMaxLen>()), (zt_min_blocks
   __syncthreads();
   if (inside && row < g.Lz) {  // t line (column, z = row): forward, factor, inverse
     const int y = quot(q, g.x), x = q - y * g.Lx;
-    float a = 0.f;
-    if constexpr (sizeof(T) == 4) a = __ldg(s2p + x) + __ldg(s2p + kMaxL + y) + __ldg(s2p + 2 * kMaxL + row);
+    df a = {0.f, 0.f}, c = a;
+    if constexpr (sizeof(T) == 4) {
+      a = p2_xyz(s2p, x, y, row);
+      c = {c_over_V, __ldg(s2p + kCLow)};
+    }
     with_length<kMaxLen>(g.Lt, [&](auto n) {
-      t_line<decltype(n)::value, T>(tile + row * g.bx + xb, g.PT, a, (q | row) == 0, c_over_V,
+      t_line<decltype(n)::value, T>(tile + row * g.bx + xb, g.PT, a, (q | row) == 0, c,
                                     kfac + (q + g.S * row), g.S * g.Lz);
     });
   }

@@ -21,7 +21,7 @@ cudaError_t pair_init() {
   constexpr int BX = pair_bx(LZ > LT ? LZ : LT);
   constexpr size_t sm = zt_smem_bytes<float, LZ, LT, BX>();
   if constexpr (sm > 48 * 1024)
-    return cudaFuncSetAttribute(k_plane_zt<LZ, LT, BX, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    return cudaFuncSetAttribute(k_plane_zt<LZ, LT, BX, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   return cudaSuccess;
 }
 
@@ -31,7 +31,7 @@ cudaError_t pair_launch(void* D, int Lx, int Ly, const float* s2p, float c_over_
   constexpr int BX = pair_bx(LZ > LT ? LZ : LT);
   constexpr size_t sm = zt_smem_bytes<float, LZ, LT, BX>();
   dim3 grid((unsigned)((Lx * Ly + BX - 1) / BX), 4);
-  return launch_pdl(k_plane_zt<LZ, LT, BX, 0>, grid, zt_threads<LZ, LT, BX>(), sm, s,
+  return launch_pdl(k_plane_zt<LZ, LT, BX, 0, true>, grid, zt_threads<LZ, LT, BX>(), sm, s,
                     static_cast<cx<float>*>(D), Lx, Ly, s2p, c_over_V, st);
 }
 

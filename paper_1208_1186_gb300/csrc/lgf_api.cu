@@ -62,7 +62,8 @@ struct Engine {
   int kmax_exponent = 0;  // FP64: biased exponent of kfac's largest entry
   double* s2d = nullptr;  // FP64: [4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions
   float* s2p = nullptr;  // FP32: [3][4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions of radix order 0, 1
-                         // and at the tile slots of order 2 (the pair split)
+                         // and at the tile slots of order 2 (the pair split), then the low parts of order 0's
+                         // x, y and z and, where t's would be, that of c_over_V
   float c_over_V = 0.f;  // p2_max / V
   size_t cbytes() const { return 2 * (size_t)prec; }
 };
@@ -345,7 +346,7 @@ int alloc_engine(lgf_handle h, Engine& e) {
   // acceleration factor at every position the forward passes leave a mode:
   // position p along an axis holds frequency digit_rev(L, p)
   std::vector<double> s2[4];
-  std::vector<float> s2f(3 * 4 * kMaxL, 0.0f);
+  std::vector<float> s2f(4 * 4 * kMaxL, 0.0f);  // order 0, 1, the pair split, low parts of order 0 (zt_plane.cuh)
   double p2max = 0.0;
   for (int a = 0; a < 4; ++a) {
     const int L = h->L[a];
@@ -356,6 +357,7 @@ int alloc_engine(lgf_handle h, Engine& e) {
           sinl(3.14159265358979323846264338327950288L * (long double)regfft::digit_rev(L, p) / (long double)L);
       s2[a][p] = (double)(4.0L * sk * sk);
       s2f[a * kMaxL + p] = (float)s2[a][p];
+      if (a < 3) s2f[3 * 4 * kMaxL + a * kMaxL + p] = (float)(s2[a][p] - (double)(float)s2[a][p]);
       m = s2[a][p] > m ? s2[a][p] : m;
       // the same at the positions of radix order 1
       const long double sk1 = sinl(3.14159265358979323846264338327950288L *
@@ -370,7 +372,9 @@ int alloc_engine(lgf_handle h, Engine& e) {
     }
     p2max += m;
   }
-  e.c_over_V = (float)(p2max / (double)V);
+  const double c_over_V = p2max / (double)V;
+  e.c_over_V = (float)c_over_V;
+  s2f[3 * 4 * kMaxL + 3 * kMaxL] = (float)(c_over_V - (double)e.c_over_V);
   if (e.prec == 4) {
     e.s2p = static_cast<float*>(dev_alloc(h, s2f.size() * sizeof(float)));
     if (!e.s2p) return fail(h, LGF_ERR_OOM, "device allocation failed");

@@ -6,6 +6,7 @@
 #pragma once
 
 #include "fft_reg.cuh"
+#include "lgf_df.cuh"
 #include "lgf_kernels.cuh"
 
 namespace lgf {
@@ -40,9 +41,31 @@ constexpr size_t zt_smem_bytes() {
   return (size_t)zt_pitch<T, LZ, BX>() * LT * sizeof(cx<T>);
 }
 
+// the low parts of s2p[0] (x, y, z) and of c_over_V, for factors rounded once
+constexpr int kS2Low = 3 * 4 * kMaxL;
+constexpr int kCLow = kS2Low + 3 * kMaxL;
+
+// the x, y and z terms of p2(k) as hi + lo
+__device__ __forceinline__ df p2_xyz(const float* __restrict__ s2p, int x, int y, int z) {
+  const df xy = two_sum(__ldg(s2p + x), __ldg(s2p + kMaxL + y));
+  df a = two_sum(xy.h, __ldg(s2p + 2 * kMaxL + z));
+  a.l += xy.l + (__ldg(s2p + kS2Low + x) + __ldg(s2p + kS2Low + kMaxL + y) + __ldg(s2p + kS2Low + 2 * kMaxL + z));
+  return a;
+}
+
+// p2_max / (V p2(k)) at position P of a t line (radix order 0)
+template <int LT, int P>
+__device__ __forceinline__ float factor_rounded(df c, df a) {
+  constexpr double s2 = regfft::MomentumSq<LT, P>::value;
+  constexpr float h = (float)s2, l = (float)(s2 - (double)h);
+  return df_quotient(c, a, {h, l});
+}
+
 // FP32: factor from s2p[RO][axis][position] and c_over_V = p2_max / V, 0 at
-// k = 0
-template <int LZ, int LT, int BX, int RO>
+// k = 0.  EXACT (RO 0): rounded once from hi + lo parts, 6e-8 of it, for the
+// shapes whose factor has always been formed in FP64 and rounded; the tuned
+// shapes' is formed in FP32, up to 2e-7.
+template <int LZ, int LT, int BX, int RO, bool EXACT = false>
 __global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), zt_min_blocks<LZ, LT, BX>())
     k_plane_zt(cx<float>* __restrict__ D, int Lx, int Ly, const float* __restrict__ s2p, float c_over_V,
                const DevState* __restrict__ st) {
@@ -86,15 +109,23 @@ __global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), zt_min_blocks<LZ, LT
     regfft::forward<T, LT, RO>(v);
     const int q = q0 + xb, y = q / Lx, x = q - y * Lx;
     // the t contribution at each position is a compile-time constant
-    const float a = __ldg(s2p + x) + __ldg(s2p + kMaxL + y) + __ldg(s2p + RO * 4 * kMaxL + 2 * kMaxL + z);
     const bool origin = (x | y | z) == 0;
-    regfft::static_for<0, LT>([&](auto pc) {
-      constexpr int p = decltype(pc)::value;
-      constexpr float s2t = (float)regfft::MomentumSq<LT, p, RO>::value;
-      float kf = c_over_V * rcp_approx(a + s2t);
-      if (p == 0 && origin) kf = 0.0f;
-      v[p] = scale(v[p], (T)kf);
-    });
+    if constexpr (EXACT) {
+      const df a = p2_xyz(s2p, x, y, z), c = {c_over_V, __ldg(s2p + kCLow)};
+      regfft::static_for<0, LT>([&](auto pc) {
+        constexpr int p = decltype(pc)::value;
+        v[p] = scale(v[p], p == 0 && origin ? 0.0f : factor_rounded<LT, p>(c, a));
+      });
+    } else {
+      const float a = __ldg(s2p + x) + __ldg(s2p + kMaxL + y) + __ldg(s2p + RO * 4 * kMaxL + 2 * kMaxL + z);
+      regfft::static_for<0, LT>([&](auto pc) {
+        constexpr int p = decltype(pc)::value;
+        constexpr float s2t = (float)regfft::MomentumSq<LT, p, RO>::value;
+        float kf = c_over_V * rcp_approx(a + s2t);
+        if (p == 0 && origin) kf = 0.0f;
+        v[p] = scale(v[p], (T)kf);
+      });
+    }
     regfft::inverse<T, LT, RO>(v);
 #pragma unroll
     for (int p = 0; p < LT; ++p) line[p * PT] = v[p];
