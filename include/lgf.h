@@ -348,8 +348,9 @@ int lgf_batch_autotune(lgf_batch b, int reps, int* lanes_out);
  * the handle's engines, reps Fourier accelerations each, and use the fastest
  * from now on (unless LGF_FFT_PIPELINE forces a pipeline).  The schedules
  * are the pipelines (x-y/z-t register planes, per-axis register passes,
- * planes of any extents) and, for the register planes, the x-run
- * width of the z-t tiles (4 or 8 FP32 complex numbers, 2 or 4 FP64) and
+ * planes of any extents; FP64 runs both kinds of planes by the same kernels,
+ * which are timed once) and, for the register planes, the x-run width of the
+ * z-t tiles (4 or 8 FP32 complex numbers) and
  * the radix order of the z and t transforms (0: radix 4 first, 32 = 4 4 2;
  * 1: the same factors reversed, 32 = 2 4 4; FP32 only, where the stages
  * differ; 2: the pair split, FP32 lines of even length with one extent of

@@ -860,12 +860,16 @@ int tune_engine(lgf_handle h, Engine& e, int reps, TuneEntry* out) {
     }
   }
   LGF_CUDA(h, cudaMemsetAsync(e.D, 0, (size_t)4 * h->V * e.cbytes(), h->stream));
+  // (FP64 runs pipelines 1 and 3 and every tile width by the same kernels: the
+  // default one of them stands for all)
   std::vector<TuneEntry> cands;
-  cands.push_back({1, 0, 0});
+  if (e.prec == 8)
+    cands.push_back({e.plane ? 3 : 1, 0, 0});
+  else
+    cands.push_back({1, 0, 0});
   if (e.axis) cands.push_back({2, 0, 0});
-  if (e.plane) {
-    const int b0 = e.prec == 4 ? 4 : 2;
-    for (int bx : {0, 2 * b0})
+  if (e.plane && e.prec == 4) {
+    for (int bx : {0, 8})
       for (int ro : {0, 1, 2})
         if (plane_zt_schedule_supported(e.prec, h->L[0], h->L[2], h->L[3], bx, ro)) cands.push_back({3, bx, ro});
   }

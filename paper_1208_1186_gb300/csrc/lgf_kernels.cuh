@@ -134,8 +134,8 @@ cudaError_t launch_plane_xy(int L, void* D, int64_t V, int Lz, int Lt, int inver
 // FP32 z-t pass schedule: bx = x-run width of a tile (0: the default, 4; or 8),
 // ro = radix order of the z and t transforms; s2p holds [3][4][kMaxL] momenta and
 // the low parts of the first block's (Engine::s2p).
-// FP64 takes bx = 0, 2 or 4 and ro = 0: its pass (fft_fx.cuh) has a tiling of
-// its own, and every schedule runs the same kernels.
+// FP64 accepts bx = 0, 2 or 4 and ro = 0, as saved schedules have them: its pass
+// (fft_fx.cuh) has a tiling of its own, and every schedule runs the same kernels.
 bool plane_zt_schedule_supported(int prec, int Lx, int Lz, int Lt, int bx, int ro);
 cudaError_t launch_plane_zt(int Lx, int Ly, int Lz, int Lt, void* D, const float* s2p, float c_over_V, int bx, int ro,
                             const DevState* st, cudaStream_t s);
