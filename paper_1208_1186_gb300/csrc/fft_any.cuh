@@ -17,7 +17,7 @@
 #pragma once
 
 #include "fft_any_geom.cuh"
-#include "zt_plane.cuh"
+#include "fft_reg.cuh"
 
 namespace lgf {
 namespace anyfft {
@@ -74,10 +74,19 @@ __device__ __noinline__ void x_line(cx<T>* row) {
   for (int i = 0; i < L; ++i) row[i] = v[i];
 }
 
-// forward t, times the acceleration factor, inverse t.  FP32: c / (a + s2t),
-// rounded once, 0 at the origin; FP64: the table at kl, step apart.
+// forward t, times the acceleration factor (the table at kl, step apart),
+// inverse t
 template <int L, class T>
-__device__ __noinline__ void t_line(cx<T>* line, int PT, df a, bool origin, df c, const T* kl, int step) {
+__device__ __noinline__ void t_line(cx<T>* line, int PT, const T* kl, int step) {
+  constexpr bool kAhead = sizeof(T) == 4;  // FP32 lines leave registers for the factors: loaded before the transform
+  T k[kAhead ? L : 1];
+  if constexpr (kAhead) {
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      k[i] = __ldg(kl);
+      kl += step;
+    }
+  }
   cx<T> v[L];
   cx<T>* p = line;
 #pragma unroll
@@ -86,14 +95,11 @@ __device__ __noinline__ void t_line(cx<T>* line, int PT, df a, bool origin, df c
     p += PT;
   }
   regfft::forward<T, L>(v);
-  if constexpr (sizeof(T) == 4) {
-    regfft::static_for<0, L>([&](auto pc) {
-      constexpr int i = decltype(pc)::value;
-      v[i] = scale(v[i], (T)(i == 0 && origin ? 0.0f : factor_rounded<L, i>(c, a)));
-    });
-  } else {
 #pragma unroll
-    for (int i = 0; i < L; ++i) {
+  for (int i = 0; i < L; ++i) {
+    if constexpr (kAhead) {
+      v[i] = scale(v[i], k[i]);
+    } else {
       v[i] = scale(v[i], __ldg(kl));
       kl += step;
     }
@@ -172,12 +178,10 @@ constexpr int zt_min_blocks() {
 // columns of a (z, t) site are contiguous, and a run may cross from one y to
 // the next.  z lines come from global memory into registers, go to the t lines
 // through shared memory, and are stored from registers after the inverse.
-// FP32: the factor from s2p and c_over_V as in k_plane_zt (EXACT); FP64: the
-// per-site table kfac.
+// The factor comes from the per-site table kfac.
 template <class T, int kMaxLen>
 __global__ void __launch_bounds__((zt_max_threads<T, kMaxLen>()), (zt_min_blocks<T, kMaxLen>()))
-    k_any_zt(cx<T>* __restrict__ D, const ZtGeom g, const T* __restrict__ kfac, const float* __restrict__ s2p,
-             float c_over_V, const DevState* __restrict__ st) {
+    k_any_zt(cx<T>* __restrict__ D, const ZtGeom g, const T* __restrict__ kfac, const DevState* __restrict__ st) {
   pdl_wait();
   if (st != nullptr && st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -193,15 +197,8 @@ __global__ void __launch_bounds__((zt_max_threads<T, kMaxLen>()), (zt_min_blocks
     });
   __syncthreads();
   if (inside && row < g.Lz) {  // t line (column, z = row): forward, factor, inverse
-    const int y = quot(q, g.x), x = q - y * g.Lx;
-    df a = {0.f, 0.f}, c = a;
-    if constexpr (sizeof(T) == 4) {
-      a = p2_xyz(s2p, x, y, row);
-      c = {c_over_V, __ldg(s2p + kCLow)};
-    }
     with_length<kMaxLen>(g.Lt, [&](auto n) {
-      t_line<decltype(n)::value, T>(tile + row * g.bx + xb, g.PT, a, (q | row) == 0, c,
-                                    kfac + (q + g.S * row), g.S * g.Lz);
+      t_line<decltype(n)::value, T>(tile + row * g.bx + xb, g.PT, kfac + (q + g.S * row), g.S * g.Lz);
     });
   }
   __syncthreads();
@@ -238,10 +235,10 @@ cudaError_t Zt<T, kMaxLen>::init(int smem) {
 
 template <class T, int kMaxLen>
 cudaError_t Zt<T, kMaxLen>::launch(void* D, const ZtGeom& g, size_t smem, int threads, const void* kfac,
-                                   const float* s2p, float c_over_V, const DevState* st, cudaStream_t s) {
+                                   const DevState* st, cudaStream_t s) {
   const dim3 grid((unsigned)((g.S + g.bx - 1) / g.bx), 4);
   return launch_pdl(k_any_zt<T, kMaxLen>, grid, threads, smem, s, static_cast<cx<T>*>(D), g,
-                    static_cast<const T*>(kfac), s2p, c_over_V, st);
+                    static_cast<const T*>(kfac), st);
 }
 
 }  // namespace anyfft

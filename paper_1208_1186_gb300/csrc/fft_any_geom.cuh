@@ -21,11 +21,10 @@ struct XyGeom {
 };
 
 struct ZtGeom {
-  int Lx, Ly, Lz, Lt;
+  int Lz, Lt;
   int S, V;       // Lx Ly columns, sites
   int bx, lbx;    // columns per tile (a power of two) and its logarithm
   int PT;         // padded t pitch of a tile
-  Div x;          // by Lx
 };
 
 constexpr int kXyThreads = 128;
@@ -45,8 +44,8 @@ struct Xy {
 template <class T, int kMaxLen>
 struct Zt {
   static cudaError_t init(int smem);
-  static cudaError_t launch(void* D, const ZtGeom& g, size_t smem, int threads, const void* kfac, const float* s2p,
-                            float c_over_V, const DevState* st, cudaStream_t s);
+  static cudaError_t launch(void* D, const ZtGeom& g, size_t smem, int threads, const void* kfac, const DevState* st,
+                            cudaStream_t s);
 };
 
 }  // namespace anyfft

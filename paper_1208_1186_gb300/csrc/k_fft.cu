@@ -39,13 +39,10 @@ XyGeom xy_geom(int prec, const int L[4], size_t* smem) {
 // more where the z and t lines are short, as long as two CTAs per SM remain.
 ZtGeom zt_geom(int prec, const int L[4], size_t* smem, int* threads) {
   ZtGeom g;
-  g.Lx = L[0];
-  g.Ly = L[1];
   g.Lz = L[2];
   g.Lt = L[3];
   g.S = L[0] * L[1];
   g.V = g.S * L[2] * L[3];
-  g.x = anyfft::make_div(g.Lx);
   const int m = g.Lz > g.Lt ? g.Lz : g.Lt;
   g.bx = prec == 4 ? 4 : 2;
   while (2 * g.bx * m <= 128 && 4 * ((g.S + 2 * g.bx - 1) / (2 * g.bx)) >= 2 * kSms) g.bx *= 2;
@@ -60,23 +57,28 @@ ZtGeom zt_geom(int prec, const int L[4], size_t* smem, int* threads) {
   return g;
 }
 
-// the FP64 acceleration factor of every site, in the positions the forward
-// passes leave the modes (an FP64 division per mode and iteration would cost
-// more than reading it)
-__global__ void __launch_bounds__(256) k_kfac(const double* __restrict__ s2, double p2max, double* __restrict__ kfac,
-                                              int Lx, int Ly, int Lz, int V) {
+// the acceleration factor of every site, formed in FP64, in the positions the
+// forward passes leave the modes (an FP64 division per mode and iteration would
+// cost more than reading it)
+template <class T>
+__global__ void __launch_bounds__(256) k_kfac(const double* __restrict__ s2, double p2max, T* __restrict__ kfac, int Lx,
+                                              int Ly, int Lz, int V) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= V) return;
   const int x = s % Lx, r = s / Lx, y = r % Ly, zt = r / Ly, z = zt % Lz, t = zt / Lz;
   const double p2 = s2[x] + s2[kMaxL + y] + s2[2 * kMaxL + z] + s2[3 * kMaxL + t];
-  kfac[s] = s ? p2max / (p2 * (double)V) : 0.0;
+  kfac[s] = s ? (T)(p2max / (p2 * (double)V)) : (T)0;
 }
 
 }  // namespace
 
-cudaError_t launch_kfac(const int L[4], const double* s2, double p2max, double* kfac, cudaStream_t s) {
+cudaError_t launch_kfac(int prec, const int L[4], const double* s2, double p2max, void* kfac, cudaStream_t s) {
   const int V = L[0] * L[1] * L[2] * L[3];
-  k_kfac<<<(unsigned)((V + 255) / 256), 256, 0, s>>>(s2, p2max, kfac, L[0], L[1], L[2], V);
+  const unsigned nb = (unsigned)((V + 255) / 256);
+  if (prec == 8)
+    k_kfac<<<nb, 256, 0, s>>>(s2, p2max, static_cast<double*>(kfac), L[0], L[1], L[2], V);
+  else
+    k_kfac<<<nb, 256, 0, s>>>(s2, p2max, static_cast<float*>(kfac), L[0], L[1], L[2], V);
   return cudaPeekAtLastError();
 }
 
@@ -141,12 +143,12 @@ cudaError_t launch_fft_xy(int prec, const int L[4], void* D, int inverse, const 
   return anyfft::Xy<float, 64>::launch(D, g, sm, inv, st, s);
 }
 
-cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, int kmax_exponent, const float* s2p,
-                          float c_over_V, const DevState* st, cudaStream_t s) {
+cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, int kmax_exponent, const DevState* st,
+                          cudaStream_t s) {
   if (zt_pair_supported(prec, L[2], L[3])) {
     switch (L[2]) {
 #define LGF_CASE(N) \
-  case N: return launch_zt_pair<N>(L[3], D, L[0], L[1], s2p, c_over_V, st, s);
+  case N: return launch_zt_pair<N>(L[3], D, L[0], L[1], static_cast<const float*>(kfac), st, s);
       LGF_PAIR_EXTENTS(LGF_CASE)
 #undef LGF_CASE
     }
@@ -158,10 +160,10 @@ cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, i
   if (prec == 8) {
     if (m <= 32)
       return fxfft::launch_zt(D, g, sm, thr, static_cast<const double*>(kfac), kmax_exponent, st, s);
-    return anyfft::Zt<double, 64>::launch(D, g, sm, thr, kfac, s2p, c_over_V, st, s);
+    return anyfft::Zt<double, 64>::launch(D, g, sm, thr, kfac, st, s);
   }
-  if (m <= 32) return anyfft::Zt<float, 32>::launch(D, g, sm, thr, kfac, s2p, c_over_V, st, s);
-  return anyfft::Zt<float, 64>::launch(D, g, sm, thr, kfac, s2p, c_over_V, st, s);
+  if (m <= 32) return anyfft::Zt<float, 32>::launch(D, g, sm, thr, kfac, st, s);
+  return anyfft::Zt<float, 64>::launch(D, g, sm, thr, kfac, st, s);
 }
 
 }  // namespace lgf

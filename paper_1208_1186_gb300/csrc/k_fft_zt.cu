@@ -151,7 +151,7 @@ cudaError_t zt_launch_one(void* D, int Lx, int Ly, const float* s2p, float c_ove
                           cudaStream_t s) {
   dim3 grid((unsigned)((Lx * Ly + BX - 1) / BX), 4);
   return launch_pdl(k_plane_zt<LZ, LT, BX, RO>, grid, zt_threads<LZ, LT, BX>(), zt_smem_bytes<float, LZ, LT, BX>(), s,
-                    static_cast<cx<float>*>(D), Lx, Ly, s2p, c_over_V, st);
+                    static_cast<cx<float>*>(D), Lx, Ly, s2p, c_over_V, nullptr, st);
 }
 
 template <int LZ, int LT, int BX>

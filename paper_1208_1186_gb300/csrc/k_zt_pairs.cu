@@ -26,13 +26,12 @@ cudaError_t pair_init() {
 }
 
 template <int LZ, int LT>
-cudaError_t pair_launch(void* D, int Lx, int Ly, const float* s2p, float c_over_V, const DevState* st,
-                        cudaStream_t s) {
+cudaError_t pair_launch(void* D, int Lx, int Ly, const float* kfac, const DevState* st, cudaStream_t s) {
   constexpr int BX = pair_bx(LZ > LT ? LZ : LT);
   constexpr size_t sm = zt_smem_bytes<float, LZ, LT, BX>();
   dim3 grid((unsigned)((Lx * Ly + BX - 1) / BX), 4);
   return launch_pdl(k_plane_zt<LZ, LT, BX, 0, true>, grid, zt_threads<LZ, LT, BX>(), sm, s,
-                    static_cast<cx<float>*>(D), Lx, Ly, s2p, c_over_V, st);
+                    static_cast<cx<float>*>(D), Lx, Ly, nullptr, 0.f, kfac, st);
 }
 
 }  // namespace
@@ -49,11 +48,10 @@ cudaError_t zt_pair_init(int Lt) {
 }
 
 template <int LZ>
-cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* s2p, float c_over_V, const DevState* st,
-                           cudaStream_t s) {
+cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* kfac, const DevState* st, cudaStream_t s) {
   switch (Lt) {
 #define LGF_CASE(LT) \
-  case LT: return pair_launch<LZ, LT>(D, Lx, Ly, s2p, c_over_V, st, s);
+  case LT: return pair_launch<LZ, LT>(D, Lx, Ly, kfac, st, s);
     LGF_PAIR_EXTENTS(LGF_CASE)
 #undef LGF_CASE
     default: return cudaErrorInvalidValue;
@@ -61,7 +59,6 @@ cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* s2p, fl
 }
 
 template cudaError_t zt_pair_init<LGF_PAIR_Z>(int);
-template cudaError_t launch_zt_pair<LGF_PAIR_Z>(int, void*, int, int, const float*, float, const DevState*,
-                                                cudaStream_t);
+template cudaError_t launch_zt_pair<LGF_PAIR_Z>(int, void*, int, int, const float*, const DevState*, cudaStream_t);
 
 }  // namespace lgf

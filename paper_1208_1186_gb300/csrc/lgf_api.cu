@@ -58,12 +58,11 @@ struct Engine {
   int zt_bx = 0;         // plane pipeline: x-run width of the z-t tiles (0: default)
   int zt_ro = 0;         // plane pipeline: radix order of the z and t transforms
   bool grep = false;     // FP32 engine: gauge representation (U holds the loaded links, G is updated)
-  void* kfac = nullptr;  // FP64: p2_max/(V p2(k)) per site, digit-reversed order
+  void* kfac = nullptr;  // p2_max/(V p2(k)) per site, digit-reversed order, formed in FP64 (FP32: planes of pipeline 1)
   int kmax_exponent = 0;  // FP64: biased exponent of kfac's largest entry
-  double* s2d = nullptr;  // FP64: [4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions
+  double* s2d = nullptr;  // [4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions
   float* s2p = nullptr;  // FP32: [3][4][kMaxL] 4 sin^2(pi k/L) at the digit-reversed positions of radix order 0, 1
-                         // and at the tile slots of order 2 (the pair split), then the low parts of order 0's
-                         // x, y and z and, where t's would be, that of c_over_V
+                         // and at the tile slots of order 2 (the pair split)
   float c_over_V = 0.f;  // p2_max / V
   size_t cbytes() const { return 2 * (size_t)prec; }
 };
@@ -346,7 +345,7 @@ int alloc_engine(lgf_handle h, Engine& e) {
   // acceleration factor at every position the forward passes leave a mode:
   // position p along an axis holds frequency digit_rev(L, p)
   std::vector<double> s2[4];
-  std::vector<float> s2f(4 * 4 * kMaxL, 0.0f);  // order 0, 1, the pair split, low parts of order 0 (zt_plane.cuh)
+  std::vector<float> s2f(3 * 4 * kMaxL, 0.0f);
   double p2max = 0.0;
   for (int a = 0; a < 4; ++a) {
     const int L = h->L[a];
@@ -357,7 +356,6 @@ int alloc_engine(lgf_handle h, Engine& e) {
           sinl(3.14159265358979323846264338327950288L * (long double)regfft::digit_rev(L, p) / (long double)L);
       s2[a][p] = (double)(4.0L * sk * sk);
       s2f[a * kMaxL + p] = (float)s2[a][p];
-      if (a < 3) s2f[3 * 4 * kMaxL + a * kMaxL + p] = (float)(s2[a][p] - (double)(float)s2[a][p]);
       m = s2[a][p] > m ? s2[a][p] : m;
       // the same at the positions of radix order 1
       const long double sk1 = sinl(3.14159265358979323846264338327950288L *
@@ -372,28 +370,25 @@ int alloc_engine(lgf_handle h, Engine& e) {
     }
     p2max += m;
   }
-  const double c_over_V = p2max / (double)V;
-  e.c_over_V = (float)c_over_V;
-  s2f[3 * 4 * kMaxL + 3 * kMaxL] = (float)(c_over_V - (double)e.c_over_V);
+  e.c_over_V = (float)(p2max / (double)V);
   if (e.prec == 4) {
     e.s2p = static_cast<float*>(dev_alloc(h, s2f.size() * sizeof(float)));
     if (!e.s2p) return fail(h, LGF_ERR_OOM, "device allocation failed");
     LGF_CUDA(h, cudaMemcpy(e.s2p, s2f.data(), s2f.size() * sizeof(float), cudaMemcpyHostToDevice));
-  } else {
-    e.kfac = dev_alloc(h, (size_t)V * e.prec);
-    e.s2d = static_cast<double*>(dev_alloc(h, (size_t)4 * kMaxL * sizeof(double)));
-    if (!e.kfac || !e.s2d) return fail(h, LGF_ERR_OOM, "device allocation failed");
-    std::vector<double> t(4 * kMaxL, 0.0);
-    for (int a = 0; a < 4; ++a) std::copy(s2[a].begin(), s2[a].end(), t.begin() + a * kMaxL);
-    LGF_CUDA(h, cudaMemcpy(e.s2d, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
-    // the largest factor is that of the smallest momentum
-    double p2min = p2max;
-    for (int a = 0; a < 4; ++a)
-      for (double s : s2[a])
-        if (s > 0.0 && s < p2min) p2min = s;
-    e.kmax_exponent = ilogb(p2max / (p2min * (double)V)) + 1023;
-    LGF_CUDA(h, launch_kfac(h->L, e.s2d, p2max, static_cast<double*>(e.kfac), h->stream));
   }
+  e.kfac = dev_alloc(h, (size_t)V * e.prec);
+  e.s2d = static_cast<double*>(dev_alloc(h, (size_t)4 * kMaxL * sizeof(double)));
+  if (!e.kfac || !e.s2d) return fail(h, LGF_ERR_OOM, "device allocation failed");
+  std::vector<double> t(4 * kMaxL, 0.0);
+  for (int a = 0; a < 4; ++a) std::copy(s2[a].begin(), s2[a].end(), t.begin() + a * kMaxL);
+  LGF_CUDA(h, cudaMemcpy(e.s2d, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
+  // the largest factor is that of the smallest momentum
+  double p2min = p2max;
+  for (int a = 0; a < 4; ++a)
+    for (double s : s2[a])
+      if (s > 0.0 && s < p2min) p2min = s;
+  e.kmax_exponent = ilogb(p2max / (p2min * (double)V)) + 1023;
+  LGF_CUDA(h, launch_kfac(e.prec, h->L, e.s2d, p2max, e.kfac, h->stream));
   return LGF_OK;
 }
 
@@ -481,7 +476,7 @@ int queue_planes_forward(lgf_handle h, Engine& e, int pipe, const DevState* st) 
                                                 s));
   } else {
     LGF_LAUNCH(h, LGF_K_FFT_XY, launch_fft_xy(e.prec, L, e.D, 0, st, s));
-    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_fft_zt(e.prec, L, e.D, e.kfac, e.kmax_exponent, e.s2p, e.c_over_V, st, s));
+    LGF_LAUNCH(h, LGF_K_FFT_ZT, launch_fft_zt(e.prec, L, e.D, e.kfac, e.kmax_exponent, st, s));
   }
   return LGF_OK;
 }

@@ -77,18 +77,6 @@ __device__ __forceinline__ df df_mul(df x, df y) {
   return fast_two_sum(p.h, __fmaf_rn(x.h, y.l, __fmaf_rn(x.l, y.h, p.l)));
 }
 
-// c / (x + y) as the nearest FP32 number but for a few 2^-48, from a reciprocal
-// within 1 ulp: q = c r with the product's remainder, corrected to first order
-// by what (x + y) r leaves of 1.  (NaN where x + y is 0.)
-__device__ __forceinline__ float df_quotient(df c, df x, df y) {
-  df p = two_sum(x.h, y.h);
-  p.l = __fadd_rn(p.l, __fadd_rn(x.l, y.l));
-  const float r = rcp_approx(p.h);
-  const float e = __fmaf_rn(-p.l, r, __fmaf_rn(-p.h, r, 1.0f));
-  const df q = two_prod(c.h, r);
-  return __fadd_rn(q.h, __fmaf_rn(q.h, e, __fmaf_rn(c.l, r, q.l)));
-}
-
 // ---------------------------------------------------------------------------
 // Compensated dot products (the Dot2 scheme of Ogita, Rump and Oishi, 2005):
 // the running sum's high part advances by exact two-sums, every product and

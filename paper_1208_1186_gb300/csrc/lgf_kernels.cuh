@@ -85,23 +85,22 @@ cudaError_t launch_unpack_fields(int prec, const void* D, double* out, int64_t V
 bool extents_supported(const int L[4], int prec, size_t smem_limit);
 cudaError_t fft_any_init(int smem);
 cudaError_t launch_fft_xy(int prec, const int L[4], void* D, int inverse, const DevState* st, cudaStream_t s);
-cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, int kmax_exponent, const float* s2p,
-                          float c_over_V, const DevState* st, cudaStream_t s);
+cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, int kmax_exponent, const DevState* st,
+                          cudaStream_t s);
 
 // FP32 z-t kernels per pair of common extents (k_zt_pairs.cu)
 #define LGF_PAIR_EXTENTS(X) \
   X(4) X(6) X(8) X(10) X(12) X(16) X(18) X(20) X(24) X(30) X(32) X(36) X(40) X(48) X(64)
 template <int LZ>
-cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* s2p, float c_over_V, const DevState* st,
-                           cudaStream_t s);
+cudaError_t launch_zt_pair(int Lt, void* D, int Lx, int Ly, const float* kfac, const DevState* st, cudaStream_t s);
 bool zt_pair_supported(int prec, int Lz, int Lt);
 // raises the shared memory limit of a pair's kernel on the current device, at
 // handle creation; for this pair alone, because touching a kernel loads it
 template <int LZ>
 cudaError_t zt_pair_init(int Lt);
 cudaError_t zt_pair_init(int Lz, int Lt);
-// kfac[s] = p2max / (V sum_a s2[a][x_a]), 0 at the origin; s2: [4][kMaxL]
-cudaError_t launch_kfac(const int L[4], const double* s2, double p2max, double* kfac, cudaStream_t s);
+// kfac[s] = p2max / (V sum_a s2[a][x_a]) in FP64 or rounded to FP32, 0 at the origin; s2: [4][kMaxL]
+cudaError_t launch_kfac(int prec, const int L[4], const double* s2, double p2max, void* kfac, cudaStream_t s);
 
 // per-axis register FFT passes (k_fft_axis.cu); lengths 4..32 (FP64) and up
 // to 64 (FP32) with radices 4, 2, 3, 5
@@ -132,8 +131,7 @@ bool plane_xy_supported(int Lx, int Ly);
 cudaError_t launch_plane_xy(int L, void* D, int64_t V, int Lz, int Lt, int inverse, const DevState* st,
                             cudaStream_t s);
 // FP32 z-t pass schedule: bx = x-run width of a tile (0: the default, 4; or 8),
-// ro = radix order of the z and t transforms; s2p holds [3][4][kMaxL] momenta and
-// the low parts of the first block's (Engine::s2p).
+// ro = radix order of the z and t transforms; s2p holds [3][4][kMaxL] momenta.
 // FP64 accepts bx = 0, 2 or 4 and ro = 0, as saved schedules have them: its pass
 // (fft_fx.cuh) has a tiling of its own, and every schedule runs the same kernels.
 bool plane_zt_schedule_supported(int prec, int Lx, int Lz, int Lt, int bx, int ro);

@@ -6,7 +6,6 @@
 #pragma once
 
 #include "fft_reg.cuh"
-#include "lgf_df.cuh"
 #include "lgf_kernels.cuh"
 
 namespace lgf {
@@ -36,39 +35,28 @@ constexpr int zt_min_blocks() {
   return LZ <= 32 && LT <= 32 ? (BX <= 4 ? 3 : 2) : 1;
 }
 
+// TABLE: the CTAs per SM that the lines' registers leave without the loads of
+// the factors, which otherwise would be kept in flight in more registers (20 x
+// 40: 148 instead of 127, two CTAs per SM for three)
+template <int LZ, int LT, int BX>
+constexpr int zt_table_min_blocks() {
+  constexpr int m = LZ > LT ? LZ : LT;
+  return m <= 24 ? zt_min_blocks<LZ, LT, BX>() : m <= 32 ? 5 : m <= 40 ? 3 : m <= 48 ? 2 : 1;
+}
+
 template <class T, int LZ, int LT, int BX>
 constexpr size_t zt_smem_bytes() {
   return (size_t)zt_pitch<T, LZ, BX>() * LT * sizeof(cx<T>);
 }
 
-// the low parts of s2p[0] (x, y, z) and of c_over_V, for factors rounded once
-constexpr int kS2Low = 3 * 4 * kMaxL;
-constexpr int kCLow = kS2Low + 3 * kMaxL;
-
-// the x, y and z terms of p2(k) as hi + lo
-__device__ __forceinline__ df p2_xyz(const float* __restrict__ s2p, int x, int y, int z) {
-  const df xy = two_sum(__ldg(s2p + x), __ldg(s2p + kMaxL + y));
-  df a = two_sum(xy.h, __ldg(s2p + 2 * kMaxL + z));
-  a.l += xy.l + (__ldg(s2p + kS2Low + x) + __ldg(s2p + kS2Low + kMaxL + y) + __ldg(s2p + kS2Low + 2 * kMaxL + z));
-  return a;
-}
-
-// p2_max / (V p2(k)) at position P of a t line (radix order 0)
-template <int LT, int P>
-__device__ __forceinline__ float factor_rounded(df c, df a) {
-  constexpr double s2 = regfft::MomentumSq<LT, P>::value;
-  constexpr float h = (float)s2, l = (float)(s2 - (double)h);
-  return df_quotient(c, a, {h, l});
-}
-
-// FP32: factor from s2p[RO][axis][position] and c_over_V = p2_max / V, 0 at
-// k = 0.  EXACT (RO 0): rounded once from hi + lo parts, 6e-8 of it, for the
-// shapes whose factor has always been formed in FP64 and rounded; the tuned
-// shapes' is formed in FP32, up to 2e-7.
-template <int LZ, int LT, int BX, int RO, bool EXACT = false>
-__global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), zt_min_blocks<LZ, LT, BX>())
+// factor from s2p[RO][axis][position] and c_over_V = p2_max / V, formed in FP32,
+// 0 at k = 0 (up to 2e-7 off).  TABLE (RO 0): from kfac, formed in FP64 and
+// rounded, for the shapes whose factor has always been.
+template <int LZ, int LT, int BX, int RO, bool TABLE = false>
+__global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), TABLE ? zt_table_min_blocks<LZ, LT, BX>()
+                                                                  : zt_min_blocks<LZ, LT, BX>())
     k_plane_zt(cx<float>* __restrict__ D, int Lx, int Ly, const float* __restrict__ s2p, float c_over_V,
-               const DevState* __restrict__ st) {
+               const float* __restrict__ kfac, const DevState* __restrict__ st) {
   using T = float;
   pdl_wait();
   if (st != nullptr && st->done) return;
@@ -110,12 +98,13 @@ __global__ void __launch_bounds__(zt_threads<LZ, LT, BX>(), zt_min_blocks<LZ, LT
     const int q = q0 + xb, y = q / Lx, x = q - y * Lx;
     // the t contribution at each position is a compile-time constant
     const bool origin = (x | y | z) == 0;
-    if constexpr (EXACT) {
-      const df a = p2_xyz(s2p, x, y, z), c = {c_over_V, __ldg(s2p + kCLow)};
-      regfft::static_for<0, LT>([&](auto pc) {
-        constexpr int p = decltype(pc)::value;
-        v[p] = scale(v[p], p == 0 && origin ? 0.0f : factor_rounded<LT, p>(c, a));
-      });
+    if constexpr (TABLE) {
+      const float* k = kfac + (q + LxLy * z);
+#pragma unroll
+      for (int p = 0; p < LT; ++p) {
+        v[p] = scale(v[p], __ldg(k));
+        k += LxLy * LZ;
+      }
     } else {
       const float a = __ldg(s2p + x) + __ldg(s2p + kMaxL + y) + __ldg(s2p + RO * 4 * kMaxL + 2 * kMaxL + z);
       regfft::static_for<0, LT>([&](auto pc) {
