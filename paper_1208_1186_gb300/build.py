@@ -18,10 +18,11 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblgf.so")
-SOURCES = ["k_links.cu", "k_links_fx.cu", "k_gauge_rep.cu", "k_fft.cu", "k_fft_any.cu", "k_fft_fx.cu", "k_zt_pairs.cu", "k_fft_axis.cu", "k_fft_plane.cu", "k_fft_zt.cu", "k_warm.cu", "k_tail.cu", "lgf_api.cu", "lgf_noalloc.cu"]
+SOURCES = ["k_links.cu", "k_links_fx.cu", "k_gauge_rep.cu", "k_fft.cu", "k_fft_any.cu", "k_fft_fx.cu", "k_fft_long.cu", "k_zt_pairs.cu", "k_fft_axis.cu", "k_fft_plane.cu", "k_fft_zt.cu", "k_warm.cu", "k_tail.cu", "lgf_api.cu", "lgf_noalloc.cu"]
 # sources compiled once per part, with -D<macro>=<part>
-PARTS = {"k_fft_any.cu": ("LGF_ANY_PART", range(3)),
+PARTS = {"k_fft_any.cu": ("LGF_ANY_PART", range(2)),
          "k_fft_fx.cu": ("LGF_FX_PART", range(5)),
+         "k_fft_long.cu": ("LGF_LONG_T", ("double", "float")),
          "k_zt_pairs.cu": ("LGF_PAIR_Z", (4, 6, 8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 64))}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

@@ -1,19 +1,18 @@
-// Fourier acceleration of any accepted extents (products of 2, 3 and 5 up to
-// 64) in three streaming passes with in-register line FFTs (fft_reg.cuh):
+// FP32 plane passes of any accepted extents (products of 2, 3 and 5 up to 64) with
+// in-register line FFTs (fft_reg.cuh), for the shapes that have no kernel of their
+// own (k_fft.cu chooses):
 //
 //   k_any_xy(fwd) -> k_any_zt (fwd z, fwd t, x p2_max/(V p2), inv t, inv z)
 //   -> k_any_xy(inv)
 //
-// the paper's "2D plus 2D" split (Sec. 2.2) for the shapes that have no kernel
-// of their own: x-y planes of unequal extents, and z-t planes beyond the common
-// extents (k_fft_plane.cu, k_fft_zt.cu and k_zt_pairs.cu have the others).  The
-// extents are run-time values, and each line's transform, whose length is a
-// template constant, is picked by a switch that is uniform over the CTA.  Only
-// the index arithmetic is run-time; it goes by multiply-high reciprocals.
+// the paper's "2D plus 2D" split (Sec. 2.2).  The extents are run-time values, and
+// each line's transform, whose length is a template constant, is picked by a
+// switch that is uniform over the CTA.  Only the index arithmetic is run-time; it
+// goes by multiply-high reciprocals.
 //
-// The Stockham kernels that ran these shapes before kept a line's stages in
-// shared memory with run-time radices, strides and divisions:
-// 20 x 30 x 18 x 40 in FP32 took 170 us per acceleration, now 45 (its z-t plane by k_zt_pairs.cu).
+// Staged butterflies in shared memory with run-time radices, strides and
+// divisions took 170 us per acceleration of 20 x 30 x 18 x 40, now 45 (its z-t
+// plane by k_zt_pairs.cu).
 #pragma once
 
 #include "fft_any_geom.cuh"
@@ -78,14 +77,11 @@ __device__ __noinline__ void x_line(cx<T>* row) {
 // inverse t
 template <int L, class T>
 __device__ __noinline__ void t_line(cx<T>* line, int PT, const T* kl, int step) {
-  constexpr bool kAhead = sizeof(T) == 4;  // FP32 lines leave registers for the factors: loaded before the transform
-  T k[kAhead ? L : 1];
-  if constexpr (kAhead) {
+  T k[L];  // loaded before the transform
 #pragma unroll
-    for (int i = 0; i < L; ++i) {
-      k[i] = __ldg(kl);
-      kl += step;
-    }
+  for (int i = 0; i < L; ++i) {
+    k[i] = __ldg(kl);
+    kl += step;
   }
   cx<T> v[L];
   cx<T>* p = line;
@@ -96,14 +92,7 @@ __device__ __noinline__ void t_line(cx<T>* line, int PT, const T* kl, int step) 
   }
   regfft::forward<T, L>(v);
 #pragma unroll
-  for (int i = 0; i < L; ++i) {
-    if constexpr (kAhead) {
-      v[i] = scale(v[i], k[i]);
-    } else {
-      v[i] = scale(v[i], __ldg(kl));
-      kl += step;
-    }
-  }
+  for (int i = 0; i < L; ++i) v[i] = scale(v[i], k[i]);
   regfft::inverse<T, L>(v);
   p = line;
 #pragma unroll
@@ -130,9 +119,9 @@ __device__ __noinline__ void z_line_out(const cx<T>* line, int bx, cx<T>* dst, i
 }
 
 // lines of kMaxLen complex numbers: as many CTAs as their registers leave
-template <class T, int kMaxLen>
+template <int kMaxLen>
 constexpr int xy_min_blocks() {
-  return sizeof(T) == 8 ? 1 : kMaxLen <= 32 ? 4 : 2;
+  return kMaxLen <= 32 ? 4 : 2;
 }
 
 // tpc tiles (one field of one (z, t) plane each: tile = 4 plane + field) per
@@ -142,7 +131,7 @@ constexpr int xy_min_blocks() {
 // shared memory as they came.  (The two 1D transforms commute.)  The row pitch
 // is odd, so no phase has bank conflicts.
 template <class T, bool INV, int kMaxLen>
-__global__ void __launch_bounds__(kXyThreads, (xy_min_blocks<T, kMaxLen>()))
+__global__ void __launch_bounds__(kXyThreads, (xy_min_blocks<kMaxLen>()))
     k_any_xy(cx<T>* __restrict__ D, const XyGeom g, const DevState* __restrict__ st) {
   pdl_wait();
   if (st != nullptr && st->done) return;
@@ -169,7 +158,7 @@ __global__ void __launch_bounds__(kXyThreads, (xy_min_blocks<T, kMaxLen>()))
   }
 }
 
-template <class T, int kMaxLen>
+template <int kMaxLen>
 constexpr int zt_min_blocks() {
   return kMaxLen <= 32 ? 3 : 1;
 }
@@ -180,7 +169,7 @@ constexpr int zt_min_blocks() {
 // through shared memory, and are stored from registers after the inverse.
 // The factor comes from the per-site table kfac.
 template <class T, int kMaxLen>
-__global__ void __launch_bounds__((zt_max_threads<T, kMaxLen>()), (zt_min_blocks<T, kMaxLen>()))
+__global__ void __launch_bounds__((zt_max_threads<kMaxLen>()), (zt_min_blocks<kMaxLen>()))
     k_any_zt(cx<T>* __restrict__ D, const ZtGeom g, const T* __restrict__ kfac, const DevState* __restrict__ st) {
   pdl_wait();
   if (st != nullptr && st->done) return;
@@ -196,11 +185,10 @@ __global__ void __launch_bounds__((zt_max_threads<T, kMaxLen>()), (zt_min_blocks
       y_line<decltype(n)::value, T, false>(Dq + g.S * g.Lz * row, g.S, tile + row * g.PT + xb, g.bx);
     });
   __syncthreads();
-  if (inside && row < g.Lz) {  // t line (column, z = row): forward, factor, inverse
+  if (inside && row < g.Lz)  // t line (column, z = row): forward, factor, inverse
     with_length<kMaxLen>(g.Lt, [&](auto n) {
       t_line<decltype(n)::value, T>(tile + row * g.bx + xb, g.PT, kfac + (q + g.S * row), g.S * g.Lz);
     });
-  }
   __syncthreads();
   if (inside && row < g.Lt)  // inverse z, to global memory
     with_length<kMaxLen>(g.Lz, [&](auto n) {

@@ -1,5 +1,6 @@
-// Geometry and launchers of the any-extent FFT kernels (fft_any.cuh, and
-// fft_fx.cuh for FP64 lines up to 32).
+// Geometry and launchers of the plane kernels whose extents are run-time values:
+// fft_any.cuh (FP32, a thread per line), fft_fx.cuh (FP64 lines up to 32) and
+// k_fft_long.cu (two steps a line).
 #pragma once
 
 #include "lgf_kernels.cuh"
@@ -30,12 +31,12 @@ struct ZtGeom {
 constexpr int kXyThreads = 128;
 
 // threads of a z-t CTA: bx max(Lz, Lt) at most
-template <class T, int kMaxLen>
+template <int kMaxLen>
 constexpr int zt_max_threads() {
-  return sizeof(T) == 4 ? 4 * kMaxLen : 2 * kMaxLen;
+  return 4 * kMaxLen;
 }
 
-// the kernels for extents up to kMaxLen = 32 (FP32) or 64
+// the FP32 kernels for extents up to kMaxLen
 template <class T, int kMaxLen>
 struct Xy {
   static cudaError_t init(int smem);
@@ -49,6 +50,19 @@ struct Zt {
 };
 
 }  // namespace anyfft
+
+namespace longfft {
+
+// plane passes of any extents in two steps a line (k_fft_long.cu)
+template <class T>
+cudaError_t init(int smem);
+template <class T>
+cudaError_t launch_xy(void* D, const anyfft::XyGeom& g, size_t smem, bool inverse, const DevState* st, cudaStream_t s);
+template <class T>
+cudaError_t launch_zt(void* D, const anyfft::ZtGeom& g, size_t smem, const void* kfac, const DevState* st,
+                      cudaStream_t s);
+
+}  // namespace longfft
 
 namespace fxfft {
 

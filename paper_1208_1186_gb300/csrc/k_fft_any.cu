@@ -10,11 +10,8 @@ namespace anyfft {
 template struct Xy<float, 32>;
 template struct Zt<float, 32>;
 #elif LGF_ANY_PART == 1
-template struct Xy<float, 64>;
+template struct Xy<float, 40>;
 template struct Zt<float, 64>;
-#elif LGF_ANY_PART == 2
-template struct Xy<double, 64>;
-template struct Zt<double, 64>;
 #endif
 
 }  // namespace anyfft
