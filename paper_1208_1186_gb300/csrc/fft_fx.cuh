@@ -12,10 +12,16 @@
 // transform rounds each number at 53 bits, this one all of them at 62 bits below
 // the line's sum.
 //
+// The exponent is the CTA's: the tiles of an x-y CTA (fields and planes) and the
+// columns of a z-t CTA share it, so numbers far below the CTA's largest are cut off
+// at 2^-61 of it, not at their own 53 bits.
+//
 // regfft's transforms (fft_reg.cuh) run on this type as they do on float and
-// double: the same stages, order and twiddles.  Error of the whole acceleration
-// against extended precision, FP64 -> this: 8^4 3.9e-16 -> 2.6e-16, 16^4 4.8e-16 ->
-// 3.3e-16, 24^4 7.7e-16 -> 6.6e-16, 32 x 32 x 8 x 8 5.6e-16 -> 4.0e-16.
+// double: the same stages and order, with twiddles and factors of 62 bits.  Error
+// of the whole acceleration against extended precision, FP64 -> this: 8^4 3.9e-16 ->
+// 1.1e-16, 16^4 4.8e-16 -> 1.3e-16, 24^3 x 12 7.1e-16 -> 1.4e-16, 32 x 32 x 8 x 8
+// 5.6e-16 -> 1.8e-16 (with twiddles of 53 bits, some units off, and factors of 60 2.7,
+// 3.3, 5.9 and 3.8e-16).
 #pragma once
 
 #include "fft_any.cuh"
@@ -38,6 +44,24 @@ struct I {
     return r;
   }
 };
+// the constant's 62 bits, of which a double has 53
+constexpr I constant(regfft::dd c) {
+  const double S = 4611686018427387904.0, x = c.h * S;
+  const long long n = (long long)x;
+  const double r = (x - (double)n) + c.l * S;
+  return I::from(n + (long long)(r + (r < 0 ? -0.5 : 0.5)));
+}
+}  // namespace fxfft
+
+namespace regfft {
+template <>
+struct Constant<fxfft::I> {
+  static constexpr fxfft::I of(dd c) { return fxfft::constant(c); }
+};
+}  // namespace regfft
+
+namespace fxfft {
+
 __device__ __forceinline__ I operator+(I a, I b) { return I::from(a.v + b.v); }
 __device__ __forceinline__ I operator-(I a, I b) { return I::from(a.v - b.v); }
 
@@ -88,6 +112,15 @@ __device__ __forceinline__ long long from_bits(long long bits, int E, int down) 
   const unsigned long long m = (((unsigned long long)bits & 0xfffffffffffffull) | (1ull << 52)) << 8;
   const long long f = e != 0 && sh < 64 ? (long long)(m >> sh) : 0;  // subnormals count as zero
   return bits < 0 ? -f : f;
+}
+
+// a factor x >= 0 as x 2^(63 - (E - 1022)), for x < 2^(E - 1023): all of the 62 bits
+// a constant may have, because the product with a column's largest factor is all
+// that the smallest momenta, which carry most of the result, are left with
+__device__ __forceinline__ I factor(long long bits, int E) {
+  const int e = exponent(bits), sh = E - e;
+  const unsigned long long m = (((unsigned long long)bits & 0xfffffffffffffull) | (1ull << 52)) << 10;
+  return I::from(e != 0 && sh < 64 ? (long long)(m >> sh) : 0);
 }
 
 // |x| 2^(18 - (E - 1022)), rounded up to an integer
@@ -348,7 +381,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
 #pragma unroll 4
     for (int i = 0; i < g.Lt; ++i) {
       const longlong2 b = bits_at(tl + i * g.PT);
-      const I k = I::from(from_bits(__double_as_longlong(__ldg(kl + i * step)), EK, 0));
+      const I k = factor(__double_as_longlong(__ldg(kl + i * step)), EK);
       const I re = I::from(b.x) * k, im = I::from(b.y) * k;
       *reinterpret_cast<longlong2*>(tl + i * g.PT) = make_longlong2(re.v, im.v);
       m += size_of(re) + size_of(im);
@@ -364,8 +397,8 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   const int s3 = shift_for(slot[4], 44);
   if (zline) {
     any_line<NZ, true>(g.Lz, zl, g.bx, s3);
-    // the factor is k 2^-61 2^(EK - 1022), used as k 2^-62
-    const int X = E - 1022 - 61 + s0 + s1 + s2 + s3 + EK - 1022 + 1;
+    // the factor is k 2^-63 2^(EK - 1022), used as k 2^-62
+    const int X = E - 1022 - 61 + s0 + s1 + s2 + s3 + EK - 1022 - 1;
 #pragma unroll 4
     for (int i = 0; i < g.Lz; ++i) Dq[i * g.S] = out(zl[i * g.bx], X, E == 0x7ff);
   }

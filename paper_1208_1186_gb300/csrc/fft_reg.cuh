@@ -21,7 +21,8 @@
 // Twiddles W_L^m = exp(-2 pi i m / L) are compile-time constants (every
 // stage index is a template constant), so they become instruction immediates
 // or constant-bank operands: no table, no shared-memory loads, no registers.
-// Multiples of a quarter turn are exact sign/swap operations.
+// Multiples of a quarter turn are exact sign/swap operations.  The others are
+// the nearest numbers of the type.
 #pragma once
 
 #include <type_traits>
@@ -83,62 +84,78 @@ constexpr int digit_rev(int L, int p, int ro = 0) {
 }
 
 // ---------------------------------------------------------------------------
-// cos and sin of 2 pi m / L at compile time.  The angle is reduced to the first
-// octant with exact integer arithmetic (8 m = o L + rem), then a Taylor series
-// on [0, pi/4] (terms beyond x^25 / 25! are below 1e-27) gives the value to a
-// few units in the last place of double; octant symmetries give exact zeros,
-// ones and mirrored values.
+// cos and sin of 2 pi m / L at compile time, as the nearest double and what is
+// left of it (an FP64 transform is as accurate as its constants, whose errors
+// are the same in every line and do not average out).  The angle is reduced to
+// the first octant with exact integer arithmetic (8 m = o L + rem); a Taylor
+// series on [0, pi/4] in double-double (Dekker's and Knuth's error-free
+// transformations; terms beyond x^29 / 29! are below 1e-31 of it) gives the
+// value; octant symmetries give exact zeros, ones and mirrored values.
 // ---------------------------------------------------------------------------
-constexpr double kTwoPiOver8 = 0.78539816339744830961566084581987572;  // pi / 4
-
-constexpr double poly_sin(double x) {
-  double term = x, sum = x;
-  for (int n = 1; n <= 12; ++n) {
-    term *= -x * x / (double)((2 * n) * (2 * n + 1));
-    sum += term;
-  }
-  return sum;
+struct dd {
+  double h, l;
+};
+constexpr dd dd_fast(double a, double b) {  // |a| >= |b| or a = 0
+  const double s = a + b;
+  return {s, b - (s - a)};
+}
+constexpr dd dd_add(dd a, dd b) {
+  const double s = a.h + b.h, t = s - a.h;
+  return dd_fast(s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l));
+}
+constexpr dd dd_mul(dd a, dd b) {
+  const double p = a.h * b.h;
+  const double ca = 134217729.0 * a.h, cb = 134217729.0 * b.h;  // 2^27 + 1
+  const double ah = ca - (ca - a.h), bh = cb - (cb - b.h), al = a.h - ah, bl = b.h - bh;
+  const double e = ((ah * bh - p) + ah * bl + al * bh) + al * bl;
+  return dd_fast(p, e + (a.h * b.l + a.l * b.h));
+}
+constexpr dd dd_div(dd a, double n) {
+  const double q = a.h / n;
+  const dd r = dd_add(a, dd_mul({-q, 0.0}, {n, 0.0}));
+  return dd_fast(q, (r.h + r.l) / n);
 }
 
-constexpr double poly_cos(double x) {
-  double term = 1.0, sum = 1.0;
-  for (int n = 1; n <= 12; ++n) {
-    term *= -x * x / (double)((2 * n - 1) * (2 * n));
-    sum += term;
+// sin (first = 1) or cos (first = 0) of x in [0, pi/4]
+constexpr dd series(dd x, int first) {
+  const dd x2 = dd_mul(x, x);
+  dd term = first ? x : dd{1.0, 0.0}, sum = term;
+  for (int n = first + 2; n <= 29; n += 2) {
+    term = dd_div(dd_mul(term, {-x2.h, -x2.l}), (double)(n * (n - 1)));
+    sum = dd_add(sum, term);
   }
   return sum;
 }
 
 // {cos, sin} of 2 pi m / L; which = 0 for cos, 1 for sin
-constexpr double turn_cs(int m, int L, int which) {
+constexpr dd turn(int m, int L, int which) {
+  constexpr dd quarter_pi = {0.78539816339744830961566084581987572, 3.0616169978683829430e-17};
   m = ((m % L) + L) % L;
   const int e = 8 * m, o = e / L, rem = e - o * L;
-  const double phi = kTwoPiOver8 * (double)rem / (double)L;        // o pi/4 + phi
-  const double psi = kTwoPiOver8 * (double)(L - rem) / (double)L;  // (o+1) pi/4 - psi
-  const bool zero = rem == 0;
-  const double cp = zero ? 1.0 : poly_cos(phi), sp = zero ? 0.0 : poly_sin(phi);
-  const double cq = poly_cos(psi), sq = poly_sin(psi);
-  double c = 0.0, s = 0.0;
-  switch (o) {
-    case 0: c = cp; s = sp; break;
-    case 1: c = sq; s = cq; break;
-    case 2: c = -sp; s = cp; break;
-    case 3: c = -cq; s = sq; break;
-    case 4: c = -cp; s = -sp; break;
-    case 5: c = -sq; s = -cq; break;
-    case 6: c = sp; s = -cp; break;
-    default: c = cq; s = -sq; break;
-  }
-  return which == 0 ? c : s;
+  // octant o: o pi/4 + phi, or (o + 1) pi/4 - psi in the odd ones
+  const bool odd = o & 1;
+  const dd x = dd_div(dd_mul(quarter_pi, {(double)(odd ? L - rem : rem), 0.0}), (double)L);
+  // which of sine and cosine of x, and the sign, in octant o
+  const bool sine = (which == 1) == (o == 0 || o == 3 || o == 4 || o == 7);
+  const bool minus = which == 0 ? o >= 2 && o <= 5 : o >= 4;
+  const dd v = series(x, sine ? 1 : 0);
+  return minus ? dd{-v.h, -v.l} : v;
 }
+constexpr double turn_cs(int m, int L, int which) { return turn(m, L, which).h; }
+
+// a constant in type T
+template <class T>
+struct Constant {
+  static constexpr T of(dd c) { return (T)c.h; }
+};
 
 template <int L, int M>
 struct Twiddle {  // W_L^M = exp(-2 pi i M / L)
   static constexpr int m = ((M % L) + L) % L;
   static constexpr bool quarter = (4 * m) % L == 0;  // W in {1, -i, -1, i}
   static constexpr int q = quarter ? 4 * m / L : -1;
-  static constexpr double re = turn_cs(m, L, 0);
-  static constexpr double im = -turn_cs(m, L, 1);
+  static constexpr dd re = turn(m, L, 0);
+  static constexpr dd im = turn(-m, L, 1);
 };
 
 // v (wr + i wi)
@@ -158,8 +175,8 @@ __device__ __forceinline__ cx<T> mul_tw(cx<T> v) {
     else if constexpr (q == 2) return mk<T>(-v.re, -v.im);
     else return mk<T>(-v.im, v.re);
   } else {
-    constexpr T wr = (T)W::re;
-    constexpr T wi = CONJ ? (T)-W::im : (T)W::im;
+    constexpr T wr = Constant<T>::of(W::re);
+    constexpr T wi = Constant<T>::of(CONJ ? dd{-W::im.h, -W::im.l} : W::im);
     return mul_const(v, wr, wi);  // by argument-dependent lookup for a type with its own product
   }
 }
@@ -202,7 +219,7 @@ __device__ __forceinline__ void dft(cx<T>* v) {
     v[3] = d02 - d13;
   } else if constexpr (R == 3) {
     constexpr T h = (T)0.5;
-    constexpr T s = (T)turn_cs(1, 3, 1);  // sin(2 pi / 3)
+    constexpr T s = Constant<T>::of(turn(1, 3, 1));  // sin(2 pi / 3)
     const cx<T> t1 = v[1] + v[2];
     const cx<T> t2 = scale(mul_i(v[1] - v[2], !INV), s);
     const cx<T> m = v[0] - scale(t1, h);
@@ -210,8 +227,8 @@ __device__ __forceinline__ void dft(cx<T>* v) {
     v[1] = m + t2;
     v[2] = m - t2;
   } else {  // R == 5
-    constexpr T c1 = (T)turn_cs(1, 5, 0), c2 = (T)turn_cs(2, 5, 0);  // cos(2 pi / 5), cos(4 pi / 5)
-    constexpr T s1 = (T)turn_cs(1, 5, 1), s2 = (T)turn_cs(2, 5, 1);  // sin(2 pi / 5), sin(4 pi / 5)
+    constexpr T c1 = Constant<T>::of(turn(1, 5, 0)), c2 = Constant<T>::of(turn(2, 5, 0));  // cos(2 pi / 5), cos(4 pi / 5)
+    constexpr T s1 = Constant<T>::of(turn(1, 5, 1)), s2 = Constant<T>::of(turn(2, 5, 1));  // sin(2 pi / 5), sin(4 pi / 5)
     const cx<T> a1 = v[1] + v[4], b1 = v[1] - v[4];
     const cx<T> a2 = v[2] + v[3], b2 = v[2] - v[3];
     const cx<T> p1 = v[0] + scale(a1, c1) + scale(a2, c2);
