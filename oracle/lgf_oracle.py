@@ -4,8 +4,8 @@ Fourier acceleration.
 TEST INFRASTRUCTURE.  Only ``tests/``, ``__graft_entry__.smoke()`` and the CPU
 baseline / reference arm of ``bench.py`` may import this module.  The product
 library never calls it and shares no code with it: the GPU path packs the
-traceless anti-Hermitian gradient into four complex fields and runs a
-Stockham FFT; this oracle transforms each of the nine matrix entries on its
+traceless anti-Hermitian gradient into four complex fields and runs
+mixed-radix FFTs; this oracle transforms each of the nine matrix entries on its
 own with a naive, separable discrete Fourier transform, which is how the
 paper's own GPU code treats the gradient (Sec. 2.2: every element of Delta is
 transformed on its own, in place, in the structure-of-arrays layout).

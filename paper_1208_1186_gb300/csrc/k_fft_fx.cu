@@ -6,7 +6,9 @@
 // through the kernel of all lengths is not (z-t of 16^3 x 32: 53 against 72 us,
 // 16^4: 20.0 against 22.5; x-y of 32^4: 90 against 97).  Not the z-t planes of
 // equal extents from 20 on, whose z and t lines share one function there (32^4:
-// 171 us against 220 with two copies).
+// 171 us against 220 with two copies).  The list is LGF_ZT_F64 (lgf_kernels.cuh)
+// without those; it is not complete: other short pairs would gain as 16 x 32 does,
+// at a kernel each.
 #include "fft_fx.cuh"
 
 #define LGF_FX_EQUAL_WARP(X) X(4) X(6) X(8) X(10) X(12) X(16)

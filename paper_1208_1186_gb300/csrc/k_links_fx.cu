@@ -8,10 +8,11 @@
 //   k_update_fx    U_mu(x) <- g(x) U_mu(x) g(x+mu)^dag
 //   k_fx_store     pairs -> FP64 links, at the end of the queue
 //
-// Delta's Fourier acceleration stays FP64.  Links whose rows are not unit
-// vectors within 2^-7 do not fit the pairs' range: k_fx_load then stops the
-// queue with DevState::unfit and the host runs the FP64 kernels on the
-// untouched FP64 links.
+// Delta's Fourier acceleration takes and gives FP64 numbers (lines up to 32 run as
+// 64-bit integers inside, fft_fx.cuh).  Links whose rows are not unit vectors
+// within 2^-7 do not fit the pairs' range: k_fx_load then stops the queue with
+// DevState::unfit and the host runs the FP64 kernels on the untouched FP64 links,
+// as it does for tolerances below the pairs' floor and on handles without pairs.
 //
 // 32^4, us per launch, FP64 kernels -> these: update 1570 -> 281, gradient
 // 395 -> 118, g 218 -> 54; load and store of the pairs, once per queue, 180

@@ -4,9 +4,10 @@
 // count and occupancy the latter spent twice the time (24^3 x 48: 33 against 18
 // us), waiting for instructions (4.6 cycles per issue against 0.7, ncu) -- a
 // kernel of 27 KB of straight-line code is fetched ahead, a path through one of
-// many hundred KB is not.  FP32 only: the FP64 pass is bound by its pipe, and
-// the run-time kernel fills its warps better (20^4: 107 against 131 us).
-// Compiled once per z extent (build.py).
+// many hundred KB is not.  The price is code: 225 kernels make 71 MB of objects (the
+// library is 102 MB) and 5 of the 14 CPU minutes of its build.  FP32 only: FP64 planes run
+// in 64-bit block floating point (k_fft_fx.cu) or in two steps a line
+// (k_fft_long.cu).  Compiled once per z extent (build.py).
 #include "zt_plane.cuh"
 
 namespace lgf {

@@ -451,9 +451,11 @@ int reset_state(lgf_handle h, double tol, int max_iter, bool with_hist, bool sta
 // otherwise (a forced pipeline that does not apply falls back to 1):
 // 3, the FP32 plane kernels with tuned schedules, where the shape is
 // instantiated; else 1, plane passes of any extents.  The per-axis passes (2)
-// are seven launches, and every extent they take has plane kernels that beat
-// them (16 x 24 x 32 x 32: 88 against 81 us per update; 6 x 12 x 4 x 20: 27
-// against 21).  FP64 runs pipelines 1 and 3 by the same kernels.
+// are seven launches, and the extents they take have plane kernels that beat or
+// nearly match them (us per update, 2 against 1: 16 x 24 x 32 x 32 87 and 80, 6 x 12 x
+// 4 x 20 27 and 21, 4 x 64 x 32 x 24 55 and 50, 64 x 64 x 8 x 8 64 and 64; the worst of
+// fifty shapes 64 x 48 x 6 x 12, 56 and 60).  FP64 runs pipelines 1 and 3 by the
+// same kernels.
 int pick_pipeline(lgf_handle h, const Engine& e) {
   if (h->fft_pipeline == 0 && e.tuned != 0) return e.tuned;
   switch (h->fft_pipeline) {
@@ -607,7 +609,7 @@ int queue_iteration(lgf_handle h, Engine& e) {
   }
   const bool exact = h->exp_order == 0;
   if (h->fx) {
-    // plain FP64 on the links in fixed-point pairs; FP64 acceleration
+    // plain FP64 on the links in fixed-point pairs; the accelerated gradient between in FP64
     LGF_LAUNCH(h, LGF_K_GRADIENT, launch_gradient_fx(e.nc, h->Ufx, e.D, h->partial, h->geo, h->st, 1, s));
     int rc = queue_accelerate(h, e, h->st);
     if (rc) return rc;

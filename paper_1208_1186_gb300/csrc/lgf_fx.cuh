@@ -19,6 +19,13 @@
 // the third, at most 1/4, dropped.  A dot product of six terms is off by about
 // 2^-54, where six FP64 roundings leave about 2^-53.
 //
+// The resolution is absolute: an entry below 1/8 keeps fewer significant bits than
+// FP64 would.  Against 80-bit arithmetic the links after 26 updates of 32^4 are off
+// by 3.1e-16 rms (FP64 kernels 4.4e-16), 16^4 3.0 (4.2), 12 x 18 x 10 x 20 in 12-real
+// storage 3.4 (4.9); their entries below 1/8 alone 3.0 (1.6).  theta comes to rest at
+// 1e-31 to 2e-31, where FP64 links go on to 6e-33 and, near the identity, below
+// 1e-40; fixes to such tolerances run on the FP64 links (lgf_api.cu, kFxTheta).
+//
 // Range: |h| < 2^31 holds |x| < 2; rows of norm at most 1 + 2^-7 times unitary
 // matrices keep every entry below 1.75 and every accumulator below 2^62.
 #pragma once

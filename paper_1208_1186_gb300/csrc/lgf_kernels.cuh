@@ -85,6 +85,7 @@ cudaError_t launch_unpack_fields(int prec, const void* D, double* out, int64_t V
 bool extents_supported(const int L[4], int prec, size_t smem_limit);
 cudaError_t fft_any_init(int smem);
 cudaError_t launch_fft_xy(int prec, const int L[4], void* D, int inverse, const DevState* st, cudaStream_t s);
+// kmax_exponent: the biased exponent of kfac's largest entry (FP64)
 cudaError_t launch_fft_zt(int prec, const int L[4], void* D, const void* kfac, int kmax_exponent, const DevState* st,
                           cudaStream_t s);
 
@@ -109,8 +110,7 @@ cudaError_t axis_pass_init();
 cudaError_t launch_xpass(int prec, int L, void* D, int64_t V, int inverse, const DevState* st, cudaStream_t s);
 cudaError_t launch_strided(int prec, int L, void* D, int64_t V, int64_t S, int inverse, const DevState* st,
                            cudaStream_t s);
-// FP64: factor from the per-site table kfac (kmax_exponent: the biased exponent of its largest entry); FP32:
-// from s2p[axis][position]
+// FP64: factor from the per-site table kfac; FP32: from s2p[axis][position]
 // (4 sin^2 at the digit-reversed frequency) and c_over_V = p2_max / V
 cudaError_t launch_tpass(int prec, int L, void* D, int64_t V, int Lx, int Ly, const void* kfac, const float* s2p,
                          float c_over_V, const DevState* st, cudaStream_t s);
