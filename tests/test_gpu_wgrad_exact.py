@@ -34,6 +34,30 @@ def test_shapes_cover_the_stage_remainders():
     assert max(int(np.prod(d)) for d in DIMS) <= 1 << 15
 
 
+def test_null_network_is_rejected():
+    from paper_1208_1186_gb300 import _lib
+    from paper_1208_1186_gb300.build import build
+    build()
+    assert _lib.load().lgf_net_conv_weight_grad(None, 1, None, None, None, 8, 8, 8, 8, None) == _lib.LGF_ERR_ARG
+
+
+@pytest.mark.gpu
+def test_bad_arguments_are_rejected(lgf):  # noqa: F811
+    import torch
+    net = lgf.WarmStartNet(seed=1)
+    try:
+        x = torch.zeros((16, 48), dtype=torch.bfloat16, device="cuda")
+        out = torch.zeros(81 * 48 * 32, device="cuda")
+        call = net.lib.lgf_net_conv_weight_grad
+        p = x.data_ptr()
+        for layer, a, b, c, dims in [(0, p, p, out.data_ptr(), (2, 2, 2, 2)), (4, p, p, out.data_ptr(), (2, 2, 2, 2)),
+                                     (1, None, p, out.data_ptr(), (2, 2, 2, 2)), (1, p, p, None, (2, 2, 2, 2)),
+                                     (1, p, p, out.data_ptr(), (1, 2, 2, 2)), (1, p, p, out.data_ptr(), (2, 2, 2, 65))]:
+            assert call(net.n, layer, a, b, c, *dims, None) == lgf._lib.LGF_ERR_ARG
+    finally:
+        net.close()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("layer", [1, 2, 3])
 @pytest.mark.parametrize("dims", DIMS)
