@@ -37,7 +37,10 @@ constexpr int zt_min_blocks() {
 
 // TABLE: the CTAs per SM that the lines' registers leave without the loads of
 // the factors, which otherwise would be kept in flight in more registers (20 x
-// 40: 148 instead of 127, two CTAs per SM for three)
+// 40: 148 instead of 127, two CTAs per SM for three).  us with the factor formed in
+// FP32 and from the table: 18 x 40 16.6 and 17.1, 20 x 40 12.6 and 12.4, 10 x 24 7.9
+// and 7.8, 30 x 10 12.4 and 12.4; lines of 36 lose a CTA, 24 x 36 13.6 and 17.1 (held
+// to four they spill: 18 x 36 10.6, 10.9 and 14).
 template <int LZ, int LT, int BX>
 constexpr int zt_table_min_blocks() {
   constexpr int m = LZ > LT ? LZ : LT;
